@@ -1,0 +1,51 @@
+"""Consecutive steps overlap on the stream (a step starts while the one before it drains): the
+fields must be those of steps that are waited for one by one, and of captured steps replayed."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from paper_2101_11107_gb300 import inputs as I  # noqa: E402
+from paper_2101_11107_gb300 import lbm  # noqa: E402
+
+
+@pytest.mark.parametrize("config", [0, 2, 4, 5, 7])
+@pytest.mark.parametrize("scheme,storage", [("esoteric", "fp32"), ("ab", "fp32"), ("ab", "bf16"), ("esoteric", "fp16")])
+@pytest.mark.parametrize("edge", [48, 96])
+def test_overlapped_steps_equal_waited_steps(edge, scheme, storage, config):
+    g = I.aneurysm(7, edge=edge, period=200.0, reynolds=40.0)
+    a, b = (lbm.Domain.from_geometry(g, scheme=scheme, storage=storage) for _ in range(2))
+    for d in (a, b):
+        d.set_launch_config(config)
+    a.step(60)
+    for _ in range(60):
+        b.step(1)
+        b.sync()
+    (ra, ua), (rb, ub) = a.macroscopic(), b.macroscopic()
+    assert np.isfinite(ua).all() and np.abs(ua).max() > 0
+    assert np.array_equal(ra, rb) and np.array_equal(ua, ub)
+
+
+@pytest.mark.parametrize("scheme", ["esoteric", "ab"])
+def test_captured_steps_replay(scheme):
+    """Two steps captured in a CUDA graph on the domain's stream, replayed ten times."""
+    g = I.pipe(20, 20, 16, 8.0, tau=0.6, g0=(0.0, 0.0, 1e-5), bouzidi=True)
+    s = torch.cuda.Stream()
+    a = lbm.Domain.from_geometry(g, scheme=scheme, stream=s)
+    b = lbm.Domain.from_geometry(g, scheme=scheme)
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=s):
+        a.step(2)
+    with torch.cuda.stream(s):
+        for _ in range(10):
+            graph.replay()
+    s.synchronize()
+    b.step(20)
+    (ra, ua), (rb, ub) = a.macroscopic(), b.macroscopic()
+    assert np.abs(ua).max() > 0
+    assert np.array_equal(ra, rb) and np.array_equal(ua, ub)
