@@ -369,15 +369,15 @@ __device__ __forceinline__ void store_et(void* pop, uint32_t n, const uint32_t (
 // u has no tangential part, f_eq_i - f_eq_opp(i) = 6 w_i rho u.n.  Then the tangential momentum
 // is zeroed by d_i += c_it D_t / 6, D_t = -sum_j c_jt d_j, which leaves mass and normal
 // momentum unchanged.
-__device__ __forceinline__ void close_open(float (&d)[Q], int kind, int axis, int sgn, float phi, float U,
-                                           float rho_out, float drho_out)
+template <int AXIS, int SGN>
+__device__ __forceinline__ void close_face(float (&d)[Q], int kind, float phi, float U, float rho_out, float drho_out)
 {
+    auto normal = [](int i) { return SGN * (AXIS == 0 ? cx_of(i) : AXIS == 1 ? cy_of(i) : cz_of(i)); };
     float D = 0.0f;
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-        const int cn = sgn * (axis == 0 ? cx_of(i) : axis == 1 ? cy_of(i) : cz_of(i));
-        if (cn == 0) D += d[i];
-        if (cn < 0) D += 2.0f * d[i];
+        if (normal(i) == 0) D += d[i];
+        if (normal(i) < 0) D += 2.0f * d[i];
     }
     float rho, un;
     if (kind == KIND_INLET) {
@@ -389,13 +389,11 @@ __device__ __forceinline__ void close_open(float (&d)[Q], int kind, int axis, in
     }
     const float ru6 = 6.0f * rho * un;
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        const int cn = sgn * (axis == 0 ? cx_of(i) : axis == 1 ? cy_of(i) : cz_of(i));
-        if (cn == 1) d[i] = d[Q - 1 - i] + w_of(i) * ru6;
-    }
+    for (int i = 0; i < Q; ++i)
+        if (normal(i) == 1) d[i] = d[Q - 1 - i] + w_of(i) * ru6;
 #pragma unroll
     for (int t = 0; t < 3; ++t) {
-        if (t == axis) continue;
+        if (t == AXIS) continue;
         float mom = 0.0f;
 #pragma unroll
         for (int j = 0; j < Q; ++j) {
@@ -406,22 +404,45 @@ __device__ __forceinline__ void close_open(float (&d)[Q], int kind, int axis, in
         const float corr = -mom * (1.0f / 6.0f);
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
-            const int cn = sgn * (axis == 0 ? cx_of(i) : axis == 1 ? cy_of(i) : cz_of(i));
             const int ct = t == 0 ? cx_of(i) : t == 1 ? cy_of(i) : cz_of(i);
-            if (cn == 1 && ct != 0) d[i] += ct == 1 ? corr : -corr;
+            if (normal(i) == 1 && ct != 0) d[i] += ct == 1 ? corr : -corr;
         }
     }
 }
 
-// Wall rules on top of the bounce-back already in d (Sec. 2.1.4 in pull form, beta = opp(alpha)
+// One instance per face: the lanes of a warp that meet open cells meet one face's, and step through about
+// 90 instructions; with the face as run-time selects in one body they were about 450, on the longest path
+// of the step of a small domain.
+__device__ __forceinline__ void close_open(float (&d)[Q], int kind, int axis, int sgn, float phi, float U,
+                                           float rho_out, float drho_out)
+{
+    switch (2 * axis + (sgn > 0)) {
+    case 0: close_face<0, -1>(d, kind, phi, U, rho_out, drho_out); break;
+    case 1: close_face<0, 1>(d, kind, phi, U, rho_out, drho_out); break;
+    case 2: close_face<1, -1>(d, kind, phi, U, rho_out, drho_out); break;
+    case 3: close_face<1, 1>(d, kind, phi, U, rho_out, drho_out); break;
+    case 4: close_face<2, -1>(d, kind, phi, U, rho_out, drho_out); break;
+    default: close_face<2, 1>(d, kind, phi, U, rho_out, drho_out); break;
+    }
+}
+
+// Interpolated bounce-back on top of the bounce-back already in d (Sec. 2.1.4 in pull form, beta = opp(alpha)
 // pointing into the wall):
 //   q <  1/2: f_a(x) = 2q f*_b(x) + (1 - 2q) f*_b(x + c_a)  [= the value pulled for b]
 //   q >= 1/2: f_a(x) = f*_b(x)/(2q) + (2q - 1)/(2q) f*_a(x)
-// with halfway bounce-back kept if x + c_a is not fluid in the first branch; then the open
-// boundaries.  f*_a(x, n - 1) comes from the cell's own slot (A-B) or from the side buffer
-// (twist: that slot is the one x + c_a pulls and overwrites in this step).  Returns the mask of
-// the q >= 1/2 links, whose f*_a the twist must keep in the side buffer.
-// Position of wall link i of a Bouzidi cell in the packed link lists (q, and the twist side
+// with halfway bounce-back kept if x + c_a is not fluid in the first branch.  f*_a(x, n - 1) comes from
+// the cell's own slot (A-B) or from the side buffer (twist: that slot is the one x + c_a pulls and
+// overwrites in this step).  Explicit roundings: every kernel gives the same bits.
+__device__ __forceinline__ float wall_low(float k, float fb, float fb_pulled)
+{
+    return __fmaf_rn(k, fb, __fmul_rn(__fadd_rn(1.0f, -k), fb_pulled));
+}
+__device__ __forceinline__ float wall_high(float k, float fb, float fa)
+{
+    return __fmaf_rn(__fadd_rn(1.0f, -k), fa, __fmul_rn(k, fb));
+}
+
+// Position of wall link i of a Bouzidi cell in the packed link lists (coefficients, and the twist side
 // buffer): the cell's entries start at its aux record and follow the set bits of its wall mask
 // in direction order.
 __device__ __forceinline__ uint32_t link_index(uint32_t off, uint32_t wm, int i)
@@ -429,6 +450,18 @@ __device__ __forceinline__ uint32_t link_index(uint32_t off, uint32_t wm, int i)
     return off + (uint32_t)__popc(wm & ((1u << i) - 1u));
 }
 
+// The open-boundary closure of a cell, if it is an inlet or outlet cell (aux: its record).
+__device__ __forceinline__ void open_rules(const DomainView& v, uint32_t word, int64_t rec, const LevelArgs& a,
+                                           float (&d)[Q])
+{
+    const int kind = (int)((word >> WORD_KIND_SHIFT) & 3u);
+    if (kind >= KIND_INLET && LBM_IN_RANGE(rec, v.n_io, 6))
+        close_open(d, kind, v.io_axis[rec], v.io_sign[rec], v.io_phi[rec], a.U, a.rho_out, a.drho_out);
+}
+
+// The wall rules and closures of one cell by its own thread (the two-cell step and the kernels that only
+// read; the one-cell steps share a warp's links out among its lanes, BouzidiLinks).  Returns the mask
+// of the q >= 1/2 links, whose f*_a the twist must keep in the side buffer.
 // aux: the cell's record (v.aux[slot]) when the caller has loaded it already, else -1
 template <int ST, int SCHEME>
 __device__ __forceinline__ uint32_t wall_rules(const DomainView& v, const void* src_ab, uint32_t slot,
@@ -464,22 +497,17 @@ __device__ __forceinline__ uint32_t wall_rules(const DomainView& v, const void* 
 #pragma unroll
             for (int j = 0; j < GS; ++j) {
                 const int i = GS * g + j;
-                const float q = qg[j], fa = fg[j];
-                if (q > 0.0f) {  // 0: no link (or halfway bounce-back on this link)
-                    if (q < 0.5f) {
-                        if (!(wm & (1u << (Q - 1 - i)))) d[i] = 2.0f * q * d[i] + (1.0f - 2.0f * q) * d[Q - 1 - i];
-                    } else {
-                        const float inv2q = 0.5f / q;
-                        d[i] = inv2q * d[i] + (1.0f - inv2q) * fa;
-                        half |= 1u << i;
-                    }
+                const float k = qg[j];
+                if (k > 0.0f) {  // 0: no link (or halfway bounce-back on this link)
+                    if (!(wm & (1u << (Q - 1 - i)))) d[i] = wall_low(k, d[i], d[Q - 1 - i]);
+                } else if (k < 0.0f) {
+                    d[i] = wall_high(-k, d[i], fg[j]);
+                    half |= 1u << i;
                 }
             }
         }
     } else if (kind >= KIND_INLET) {
-        const int64_t rec = aux >= 0 ? aux : v.aux[slot];
-        if (LBM_IN_RANGE(rec, v.n_io, 6))
-            close_open(d, kind, v.io_axis[rec], v.io_sign[rec], v.io_phi[rec], a.U, a.rho_out, a.drho_out);
+        open_rules(v, word, aux >= 0 ? aux : v.aux[slot], a, d);
     }
     return half;
 }
@@ -970,69 +998,174 @@ __device__ __forceinline__ void gather(const DomainView& v, const void* src, uin
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Bouzidi links of a warp's cells, shared out among its lanes: the links of a half-brick are one run of the
+// packed list, so a lane takes entry k0 + lane, + 32, ...: code and coefficient (coalesced, before
+// pdl_wait: they never change), f*_a of the q >= 1/2 links (coalesced from the side buffer).  The cells'
+// values go through the warp's exchange area, sm[i * STRIDE + cell]: Bouzidi cells put their 27 values there,
+// the lanes apply their links in place (a link writes f_a and reads f_b only if b has no link, so the
+// order does not matter), and the cells take them back; after the collision the cells put their stored
+// values there, from which the lanes keep f*_a.  About 60 instructions a cell and 25 per 32 links, and one
+// memory latency, against 27 directions x (test, position, two predicated loads, mix) in three groups
+// of a latency each when every cell handled its own links; a boundary half-brick has 50 to 100 links.
+// Per step, before -> after: 256^3 aneurysm FP32 11.9 -> 11.0 us, 2.7 M cell Bouzidi pipe 133.5 -> 128.8 us,
+// 25 k cell TRT aneurysm 7.7 -> 6.6 us, batch of 8 FP16 aneurysms 19.3 -> 17.1 us (with the closure by
+// face above).
+template <int ST, int SCHEME, int STRIDE>
+struct BouzidiLinks {
+    static constexpr int R = 3;  // rounds of 32 links held in registers; longer runs reload
+    uint32_t k0, k1, lane;
+    uint32_t code[R];
+    float coef[R], fa[R];
+
+    __device__ __forceinline__ bool any() const { return k0 < k1; }
+    __device__ __forceinline__ void load(const DomainView& v, uint32_t k, uint32_t& c, float& b) const
+    {
+        const bool in = k < k1 && LBM_IN_RANGE(k, v.n_bq, 5);
+        c = in ? (uint32_t)__ldg(v.blink + k) : 0u;
+        b = in ? __ldg(v.bq + k) : 0.0f;
+    }
+    __device__ __forceinline__ void prefetch(const DomainView& v, uint32_t half_brick, uint32_t lane_)
+    {
+        lane = lane_;
+        k0 = k1 = 0u;
+        if (v.bstart) {
+            k0 = (uint32_t)__ldg(v.bstart + half_brick);
+            k1 = (uint32_t)__ldg(v.bstart + half_brick + 1);
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) load(v, k0 + 32u * r + lane, code[r], coef[r]);
+    }
+    // f*_a of a q >= 1/2 link, as stored
+    __device__ __forceinline__ float load_fa(const DomainView& v, const void* src, uint32_t slot0, uint32_t k, uint32_t c,
+                                             float b) const
+    {
+        if (!(b < 0.0f)) return 0.0f;
+        if (SCHEME == LBM_SCHEME_ESOTERIC) return Store<ST>::load_rw_h(v.side, k);
+        const uint32_t off = ((c >> 5) & 31u) * (uint32_t)v.n_slots + slot0 + (c & 31u);
+        return LBM_IN_RANGE(off, (uint64_t)Q * (uint64_t)v.n_slots, 1) ? Store<ST>::load_rw_h(src, off) : 0.0f;
+    }
+    __device__ __forceinline__ void issue(const DomainView& v, const void* src, uint32_t slot0)
+    {
+#pragma unroll
+        for (int r = 0; r < R; ++r) fa[r] = load_fa(v, src, slot0, k0 + 32u * r + lane, code[r], coef[r]);
+    }
+    __device__ __forceinline__ void mix(uint32_t c, float b, float other, float* sm) const
+    {
+        if (b == 0.0f) return;  // past the end, or halfway bounce-back
+        const uint32_t cell = c & 31u, dir = (c >> 5) & 31u;
+        float& f = sm[dir * STRIDE + cell];
+        if (b < 0.0f) {
+            // 16-bit storages: w = w_of(13) 4^-nnz, the same float as w_of of the direction
+            const float w = Store<ST>::SCALED ? __int_as_float(__float_as_int(w_of(13)) - (int)(((c >> 11) & 3u) << 24)) : 1.0f;
+            f = wall_high(-b, f, Store<ST>::SCALED ? __fmul_rn(w, other) : other);
+        } else if (!(c & (1u << 10))) {
+            f = wall_low(b, f, sm[(Q - 1 - dir) * STRIDE + cell]);
+        }
+    }
+    __device__ __forceinline__ void apply(const DomainView& v, const void* src, uint32_t slot0, float* sm)
+    {
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < R; ++r) mix(code[r], coef[r], fa[r], sm);
+        for (uint32_t k = k0 + 32u * R + lane; k < k1; k += 32u) {
+            uint32_t c;
+            float b;
+            load(v, k, c, b);
+            mix(c, b, load_fa(v, src, slot0, k, c, b), sm);
+        }
+        __syncwarp();
+    }
+    __device__ __forceinline__ void keep(const DomainView& v, const float* sm) const
+    {
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            if (coef[r] < 0.0f) Store<ST>::store_h(v.side, k0 + 32u * r + lane, sm[((code[r] >> 5) & 31u) * STRIDE + (code[r] & 31u)]);
+        for (uint32_t k = k0 + 32u * R + lane; k < k1; k += 32u) {
+            uint32_t c;
+            float b;
+            load(v, k, c, b);
+            if (b < 0.0f) Store<ST>::store_h(v.side, k, sm[((c >> 5) & 31u) * STRIDE + (c & 31u)]);
+        }
+    }
+};
+
 // One fused update of the cell at `slot` (a lane of a warp that covers half of one brick; all
-// 32 lanes must call it together: the neighbour row goes round by shuffle).
-// PDL: the kernel is launched as a programmatic dependent (not the persistent batch).
-template <int ST, int SCHEME, int COLL, int PC = -1, bool PDL = true>
+// 32 lanes must call it together: the neighbour row goes round by shuffle, the Bouzidi links are shared
+// out).  PDL: the kernel is launched as a programmatic dependent (not the persistent batch).  LINKS: the
+// domain may have Bouzidi cells; sm is then the warp's [27][32] exchange area.
+template <int ST, int SCHEME, int COLL, int PC = -1, bool PDL = true, bool LINKS = true>
 __device__ __forceinline__ void step_cell(const DomainView& v, const void* src, void* dst, const LevelArgs& a,
-                                          uint32_t slot, uint32_t lane)
+                                          uint32_t slot, uint32_t lane, float* sm)
 {
     constexpr bool X = COLL == COLL_CHM_FAST;  // deferred halving in the inverse transform
+    constexpr bool TWIST = SCHEME == LBM_SCHEME_ESOTERIC;
     const uint32_t brick = slot / BRICK_CELLS;
     const uint32_t word = __ldg(v.word + slot);
-    // the cell's record, loaded beside its word rather than after it: a Bouzidi or open cell then
-    // waits for one memory latency fewer before its link values (4 bytes per slot of traffic)
+    // the cell's record, loaded beside its word rather than after it: an open cell then waits for one
+    // memory latency fewer (4 bytes per slot of traffic)
     const int32_t auxv = __ldg(v.aux + slot);
+    BouzidiLinks<ST, SCHEME, 32> links;
+    if (LINKS) links.prefetch(v, slot / 32u, lane);
     const bool fluid = (word & WORD_FLUID) != 0u;
+    const bool bouzidi = ((word >> WORD_KIND_SHIFT) & 3u) == KIND_BOUZIDI;
     const uint32_t wm = word & WORD_WALL_MASK;
-    const uint32_t n = (uint32_t)v.n_slots;
+    const uint32_t n = (uint32_t)v.n_slots, slot0 = slot - lane;
     float d[Q];
+    uint32_t cs[8];
     LevelArgs la = a;
     if (word & WORD_OWN_TAU) set_own_rate<COLL>(la, __ldg(v.s2_cell + slot));
-    if (SCHEME == LBM_SCHEME_ESOTERIC) {
+    if (TWIST) {
         const int32_t row = __ldg(v.nb8 + brick * 8u + (lane & 7u));
-        uint32_t cs[8];
         corner_slots_shfl(row, slot, cs);
         const bool clean = PC >= 0 && __all_sync(0xffffffffu, wm == 0u);
         if (PDL) pdl_wait();
-        if (!fluid) return;
-        fetch_et<ST, true, PC>(dst, n, cs, wm, a.parity, d, clean);
-        const uint32_t half = wm ? wall_rules<ST, SCHEME>(v, nullptr, slot, word, a, d, auxv) : 0u;
-        collide_model<COLL, X>(d, la);
-        scale_out<ST, X>(d);
-        store_et<ST, PC, X, true>(dst, n, cs, a.parity, d);
-        if (half) {
-            const uint32_t off = (uint32_t)auxv;
-#pragma unroll
-            for (int i = 0; i < Q; ++i)
-                if ((half & (1u << i)) && LBM_IN_RANGE(link_index(off, wm, i), v.n_bq, 5))
-                    Store<ST>::store_h(v.side, link_index(off, wm, i), d[i]);
-        }
+        if (fluid) fetch_et<ST, true, PC>(dst, n, cs, wm, a.parity, d, clean);
     } else {
         const int32_t row = __ldg(v.nbr + brick * (uint32_t)Q + (lane < (uint32_t)Q ? lane : 0u));
         if (PDL) pdl_wait();
         fetch_ab_shfl<ST>(src, n, row, slot, wm, fluid, d);
-        if (!fluid) return;
-        if (wm) wall_rules<ST, SCHEME>(v, src, slot, word, a, d, auxv);
+    }
+    if (LINKS && links.any()) {
+        links.issue(v, src, slot0);
+        if (bouzidi)
+#pragma unroll
+            for (int i = 0; i < Q; ++i) sm[i * 32 + lane] = d[i];
+        links.apply(v, src, slot0, sm);
+        if (bouzidi)
+#pragma unroll
+            for (int i = 0; i < Q; ++i) d[i] = sm[i * 32 + lane];
+    }
+    if (fluid) {
+        open_rules(v, word, auxv, a, d);
         collide_model<COLL, X>(d, la);
         scale_out<ST, X>(d);
+        if (TWIST) {
+            store_et<ST, PC, X, true>(dst, n, cs, a.parity, d);
+        } else {
 #pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            if (!LBM_IN_RANGE((uint32_t)i * n + slot, (uint64_t)Q * n, 4)) continue;
-            Store<ST>::store_h(dst, (uint32_t)i * n + slot, d[i]);
+            for (int i = 0; i < Q; ++i)
+                if (LBM_IN_RANGE((uint32_t)i * n + slot, (uint64_t)Q * n, 4)) Store<ST>::store_h(dst, (uint32_t)i * n + slot, d[i]);
         }
+    }
+    if (LINKS && TWIST && links.any()) {
+        if (bouzidi)
+#pragma unroll
+            for (int i = 0; i < Q; ++i) sm[i * 32 + lane] = d[i];
+        links.keep(v, sm);
     }
 }
 
-template <int ST, int SCHEME, int BRICKS, int MINB, int COLL, int PC = -1>
+template <int ST, int SCHEME, int BRICKS, int MINB, int COLL, int PC = -1, bool LINKS = true>
 __global__ void __launch_bounds__(BRICKS * BRICK_CELLS, MINB)
     k_step(DomainView v, const void* src, void* dst, LevelArgs a)
 {
+    __shared__ float sm[LINKS ? BRICKS * 2 : 1][LINKS ? Q * 32 : 1];
     pdl_trigger();
     const uint32_t slot = blockIdx.x * (uint32_t)(BRICKS * BRICK_CELLS) + threadIdx.x;
     // the active slots are a multiple of 64, so this exit is taken by whole warps
     if (slot >= (uint32_t)(v.n_bricks * BRICK_CELLS)) return;
-    step_cell<ST, SCHEME, COLL, PC>(v, src, dst, a, slot, threadIdx.x & 31u);
+    step_cell<ST, SCHEME, COLL, PC, true, LINKS>(v, src, dst, a, slot, threadIdx.x & 31u, sm[LINKS ? threadIdx.x >> 5 : 0]);
 }
 
 // Esoteric-twist step with two cells per thread: lane l of a warp updates cells l and l + 32 of
@@ -1193,6 +1326,7 @@ __global__ void __launch_bounds__(BRICKS * BRICK_CELLS, MINB)
     k_step_batch(const BatchEntry* __restrict__ ent, const int64_t* __restrict__ brick_start, int n_dom,
                  const LevelArgs* __restrict__ args)
 {
+    __shared__ float sm[BRICKS * 2][Q * 32];
     pdl_trigger();
     const int64_t gslot = (int64_t)blockIdx.x * (BRICKS * BRICK_CELLS) + threadIdx.x;
     const int64_t gbrick = gslot / BRICK_CELLS;
@@ -1203,10 +1337,11 @@ __global__ void __launch_bounds__(BRICKS * BRICK_CELLS, MINB)
         if (__ldg(brick_start + mid) <= gbrick) lo = mid;
         else hi = mid - 1;
     }
-    const DomainView v = ent[lo].view;
+    const DomainView& v = ent[lo].view;
     const LevelArgs a = args[lo];
     const uint32_t slot = (uint32_t)((gbrick - __ldg(brick_start + lo)) * BRICK_CELLS) + (threadIdx.x & 63u);
-    step_cell<ST, LBM_SCHEME_ESOTERIC, COLL, PC>(v, ent[lo].pop, ent[lo].pop, a, slot, threadIdx.x & 31u);
+    step_cell<ST, LBM_SCHEME_ESOTERIC, COLL, PC>(v, ent[lo].pop, ent[lo].pop, a, slot, threadIdx.x & 31u,
+                                                 sm[threadIdx.x >> 5]);
 }
 
 // Persistent form of the batched step: one launch advances every domain `steps` steps.  The CTAs
@@ -1264,6 +1399,7 @@ __global__ void __launch_bounds__(BRICKS * BRICK_CELLS, MINB)
     const int64_t total = __ldg(brick_start + n_dom);
     const int64_t n_units = (total + BRICKS - 1) / BRICKS;
     __shared__ unsigned int next;
+    __shared__ float sm[BRICKS * 2][Q * 32];
     for (int s = 0; s < steps; ++s) {
         // units of step s are handed out by a ticket counter (tickets[s], cleared before the
         // launch), so that CTAs that finish early take more
@@ -1281,19 +1417,19 @@ __global__ void __launch_bounds__(BRICKS * BRICK_CELLS, MINB)
                     if (__ldg(brick_start + mid) <= gbrick) lo = mid;
                     else hi = mid - 1;
                 }
-                const DomainView v = ent[lo].view;
+                const DomainView& v = ent[lo].view;
                 const LevelArgs a = args[(size_t)s * n_dom + lo];
                 const uint32_t slot =
                     (uint32_t)((gbrick - __ldg(brick_start + lo)) * BRICK_CELLS) + (threadIdx.x & 63u);
                 // P0 >= 0: every member has parity P0 at step 0, so step s has parity P0 ^ (s & 1)
                 if (P0 >= 0 && ((s & 1) ^ P0) == 0)
                     step_cell<ST, LBM_SCHEME_ESOTERIC, COLL, (P0 >= 0 ? 0 : -1), false>(v, ent[lo].pop, ent[lo].pop, a, slot,
-                                                                                 threadIdx.x & 31u);
+                                                                                 threadIdx.x & 31u, sm[threadIdx.x >> 5]);
                 else if (P0 >= 0)
                     step_cell<ST, LBM_SCHEME_ESOTERIC, COLL, (P0 >= 0 ? 1 : -1), false>(v, ent[lo].pop, ent[lo].pop, a, slot,
-                                                                                 threadIdx.x & 31u);
+                                                                                 threadIdx.x & 31u, sm[threadIdx.x >> 5]);
                 else
-                    step_cell<ST, LBM_SCHEME_ESOTERIC, COLL, -1, false>(v, ent[lo].pop, ent[lo].pop, a, slot, threadIdx.x & 31u);
+                    step_cell<ST, LBM_SCHEME_ESOTERIC, COLL, -1, false>(v, ent[lo].pop, ent[lo].pop, a, slot, threadIdx.x & 31u, sm[threadIdx.x >> 5]);
             }
         }
         if (s + 1 < steps && !grid_barrier(bar, (unsigned int)(s + 1) * gridDim.x, limit_ns)) return;
@@ -1593,12 +1729,19 @@ cudaError_t launch_step_t(const DomainView& v, const void* src, void* dst, const
     const int grid = grid_for(v.n_bricks, BRICKS);
     return with_coll(a.coll, [&](auto c) {
         constexpr int C = decltype(c)::value;
-        // the twist with the default rates has one kernel per parity (constant plane indices)
+        constexpr int T = BRICKS * BRICK_CELLS;
+        // the default rates: a domain without Bouzidi cells runs without the link code and its exchange area
+        // (64x64x256 pipe FP16 19.9 us a step, 20.8 us with them), and the twist has one kernel
+        // per parity (constant plane indices)
         if constexpr (SCHEME == LBM_SCHEME_ESOTERIC && C == COLL_CHM_FAST) {
-            return launch_pdl(a.parity ? k_step<ST, SCHEME, BRICKS, MINB, C, 1> : k_step<ST, SCHEME, BRICKS, MINB, C, 0>,
-                              grid, BRICKS * BRICK_CELLS, 0, s, v, src, dst, a);
+            auto k = v.bstart ? (a.parity ? k_step<ST, SCHEME, BRICKS, MINB, C, 1> : k_step<ST, SCHEME, BRICKS, MINB, C, 0>)
+                              : (a.parity ? k_step<ST, SCHEME, BRICKS, MINB, C, 1, false> : k_step<ST, SCHEME, BRICKS, MINB, C, 0, false>);
+            return launch_pdl(k, grid, T, 0, s, v, src, dst, a);
+        } else if constexpr (C == COLL_CHM_FAST) {
+            auto k = v.bstart ? k_step<ST, SCHEME, BRICKS, MINB, C> : k_step<ST, SCHEME, BRICKS, MINB, C, -1, false>;
+            return launch_pdl(k, grid, T, 0, s, v, src, dst, a);
         } else {
-            return launch_pdl(k_step<ST, SCHEME, BRICKS, MINB, C>, grid, BRICKS * BRICK_CELLS, 0, s, v, src, dst, a);
+            return launch_pdl(k_step<ST, SCHEME, BRICKS, MINB, C>, grid, T, 0, s, v, src, dst, a);
         }
     });
 }

@@ -450,8 +450,11 @@ lbm_status lbm_create_domain(const uint8_t* mask, int32_t nx, int32_t ny, int32_
     // Packed link lists: each Bouzidi cell (in slot order) owns the entries [aux, aux + number of
     // its wall links) of the q list and of the twist side buffer, one per wall link in direction
     // order (q = 0 for a wall link without q: halfway bounce-back), so that the few links of a
-    // cell share one or two sectors.
-    std::vector<float> bq;
+    // cell share one or two sectors, and the links of a warp's cells (a half-brick) are one run of the
+    // list, which its lanes share out.
+    std::vector<float> bq, bcoef;
+    std::vector<uint16_t> blink;
+    std::vector<int32_t> bstart((size_t)n_bricks * 2 + 1, 0);
     for (size_t l = 0; l < lk.size();) {
         const int64_t s = lk[l].first;
         const uint32_t wmk = word[(size_t)s] & WORD_WALL_MASK;
@@ -466,9 +469,15 @@ lbm_status lbm_create_domain(const uint8_t* mask, int32_t nx, int32_t ny, int32_
         word[(size_t)s] |= (uint32_t)KIND_BOUZIDI << WORD_KIND_SHIFT;
         aux[(size_t)s] = (int32_t)bq.size();
         for (int i = 0; i < Q; ++i)
-            if ((wmk >> i) & 1u) bq.push_back(qq[i]);
+            if ((wmk >> i) & 1u) {
+                bq.push_back(qq[i]);
+                bcoef.push_back(bouzidi_coef(qq[i]));
+                blink.push_back((uint16_t)link_code((int)(s % 32), i, (wmk >> (Q - 1 - i)) & 1u));
+            }
+        bstart[(size_t)(s / 32) + 1] = (int32_t)bq.size();
         l = e;
     }
+    for (size_t h = 1; h < bstart.size(); ++h) bstart[h] = std::max(bstart[h], bstart[h - 1]);
     const int64_t n_blinks = (int64_t)bq.size();
 
     // ---------------------------------------------------------------- halo faces
@@ -548,6 +557,8 @@ lbm_status lbm_create_domain(const uint8_t* mask, int32_t nx, int32_t ny, int32_
     float* d_s2 = nullptr;
     int32_t* d_aux = nullptr;
     float* d_bq = nullptr;
+    uint16_t* d_blink = nullptr;
+    int32_t* d_bstart = nullptr;
     float* d_io_phi = nullptr;
     int8_t* d_io_axis = nullptr;
     int8_t* d_io_sign = nullptr;
@@ -556,7 +567,9 @@ lbm_status lbm_create_domain(const uint8_t* mask, int32_t nx, int32_t ny, int32_
     if (!st) st = upload(D, &d_word, word, "cell words");
     if (!st) st = upload(D, &d_s2, s2_cell, "cell relaxation rates");
     if (!st) st = upload(D, &d_aux, aux, "aux index");
-    if (!st) st = upload(D, &d_bq, bq, "Bouzidi q");
+    if (!st) st = upload(D, &d_bq, bcoef, "Bouzidi coefficients");
+    if (!st) st = upload(D, &d_blink, blink, "Bouzidi links");
+    if (!st) st = upload(D, &d_bstart, bstart, "Bouzidi link runs");
     if (!st) st = upload(D, &d_io_phi, io_phi, "inlet profile");
     if (!st) st = upload(D, &d_io_axis, io_axis, "open-boundary axis");
     if (!st) st = upload(D, &d_io_sign, io_sign, "open-boundary sign");
@@ -610,6 +623,8 @@ lbm_status lbm_create_domain(const uint8_t* mask, int32_t nx, int32_t ny, int32_
     v.s2_cell = d_s2;
     v.aux = d_aux;
     v.bq = d_bq;
+    v.blink = d_blink;
+    v.bstart = n_blinks ? d_bstart : nullptr;
     v.n_bq = std::max<int64_t>(n_blinks, 1);
     v.io_phi = d_io_phi;
     v.io_axis = d_io_axis;

@@ -70,6 +70,18 @@ constexpr uint32_t WORD_WALL_MASK = (1u << 27) - 1u;
 constexpr int WORD_KIND_SHIFT = 27;
 enum CellKind { KIND_PLAIN = 0, KIND_BOUZIDI = 1, KIND_INLET = 2, KIND_OUTLET = 3 };
 
+// Coefficient of a wall link of a Bouzidi cell: both branches of the interpolated bounce-back are
+// f_a(x) = k f*_b(x) + (1 - k) f', with k = 2q and f' the value pulled for b where q < 1/2, and k = 1/(2q)
+// and f' = f*_a(x) (both of the previous step) where q >= 1/2.  Stored as k, -k, or 0 for halfway
+// bounce-back (no q given).
+__host__ __device__ inline float bouzidi_coef(float q) { return q < 0.5f ? 2.0f * q : -(0.5f / q); }
+// The entry's cell in its half-brick, direction, whether the opposite direction is a wall link too (halfway
+// bounce-back then replaces the first branch), and the number of nonzero components of the direction.
+__host__ __device__ constexpr uint32_t link_code(int cell, int i, bool opp_wall)
+{
+    return (uint32_t)cell | ((uint32_t)i << 5) | ((uint32_t)opp_wall << 10) | ((uint32_t)nnz_of(i) << 11);
+}
+
 // Geometry of a domain on the device.
 struct DomainView {
     int64_t n_slots;        // population stride: 64 * (active + halo bricks)
@@ -79,9 +91,12 @@ struct DomainView {
     const uint32_t* word;   // [64 n_bricks]
     const int32_t* aux;     // [64 n_bricks] record of a Bouzidi or open-boundary cell
     const float* s2_cell;   // [64 n_bricks] second-order rate of cells with WORD_OWN_TAU
-    const float* bq;        // [n_bq] q of every wall link of the Bouzidi cells, packed per cell: cell
-                            // (aux record a, wall mask wm) owns a .. a + popc(wm) - 1 in direction
-                            // order (0: halfway bounce-back on that link)
+    const float* bq;        // [n_bq] coefficient of every wall link of the Bouzidi cells (bouzidi_coef),
+                            // packed per cell: cell (aux record a, wall mask wm) owns a .. a + popc(wm) - 1
+                            // in direction order
+    const uint16_t* blink;  // [n_bq] link_code of the entry
+    const int32_t* bstart;  // [2 n_bricks + 1] first entry of each half-brick (slots 32 h .. 32 h + 31);
+                            // NULL: no Bouzidi cells
     void* side;             // twist: [n_bq] f*_i of the previous step, same packing (storage type)
     int64_t n_bq;           // packed links (at least 1)
     const float* io_phi;    // [n_io] inflow profile factor 2 (1 - r^2/R^2)
