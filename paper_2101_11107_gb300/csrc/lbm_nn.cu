@@ -25,6 +25,8 @@
 #include <cuda_bf16.h>
 
 #include <cmath>
+#include <cstddef>
+#include <cstring>
 #include <string>
 #include <vector>
 
@@ -92,6 +94,47 @@ constexpr uint32_t CONV_SMEM = W_OFF + W_BYTES;         // 48640 B
 constexpr int CONV_CTAS_PER_SM = 4;
 constexpr int TC_WAIT_LIMIT = 1 << 22;
 
+// Programmatic dependent launch along a pass's chain of kernels (features, then convolutions, loss, weight
+// gradients, update): a kernel sets up its barriers, tensor memory and weights while the one before it
+// drains, and waits before it touches what the chain computes.  The features kernel is a plain launch,
+// so everything enqueued before the pass (weights, masks, fields) is complete when any kernel of the
+// chain starts.  What the chain computes is read with plain loads, not through the read-only path.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ float ld_f32(const float* p)
+{
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint32_t ld_u32(const uint32_t* p)
+{
+    uint32_t v;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint4 ld_u128(const void* p)
+{
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+template <class... P, class... A>
+cudaError_t launch_pdl(void (*k)(P...), dim3 grid, int block, size_t smem, cudaStream_t s, A&&... args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = dim3((unsigned)block);
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, k, P(args)...);
+}
+
 __device__ __forceinline__ uint32_t su32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 // shared-memory matrix descriptor: start address, leading (K) and stride (M/N) byte offsets,
@@ -130,8 +173,8 @@ struct DuArgs {
 template <int OUT>
 __global__ void __launch_bounds__(128)
     k_conv_tc(const __grid_constant__ CUtensorMap tin, const __nv_bfloat16* __restrict__ w, const float* __restrict__ bias,
-              int relu, const __nv_bfloat16* __restrict__ gate, void* __restrict__ out, const int4* __restrict__ slabs,
-              int n_slabs, Box b, unsigned int* __restrict__ err, DuArgs dua)
+              int relu, const __nv_bfloat16* gate, void* out, const int4* __restrict__ slabs, int n_slabs, Box b,
+              unsigned int* err, DuArgs dua)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) uint64_t bar_tma[2], bar_mma[2];
@@ -139,6 +182,7 @@ __global__ void __launch_bounds__(128)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int G = gridDim.x;
     const int J = (n_slabs - (int)blockIdx.x + G - 1) / G;  // slabs of this CTA (>= 1)
+    pdl_trigger();
     if (tid == 0) {
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
@@ -155,20 +199,24 @@ __global__ void __launch_bounds__(128)
     __syncthreads();
     // halo of slab j into buffer j & 1: padded coordinates (x0, y0, z) .. + (9, 17, 2), channels
     // 0-7 and 8-15 (issued by thread 0)
-    // (slab 0 also brings the weights: one bulk copy, already in the shared-memory layout)
+    // (the weights, one bulk copy already in the shared-memory layout, count towards slab 0's barrier)
+    auto load_weights = [&]() {
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(su32(&bar_tma[0])),
+                     "r"(2u * PLANE_BYTES + W_BYTES)
+                     : "memory");
+        asm volatile(
+            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                su32(smem + W_OFF)),
+            "l"(w), "r"(W_BYTES), "r"(su32(&bar_tma[0]))
+            : "memory");
+    };
     auto load_halo = [&](int j) {
         const int4 sl = slabs[blockIdx.x + j * G];
         uint64_t* bar = &bar_tma[j & 1];
         unsigned char* dst = smem + (j & 1) * HALO_BYTES;
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(su32(bar)),
-                     "r"(2u * PLANE_BYTES + (j == 0 ? W_BYTES : 0u))
-                     : "memory");
-        if (j == 0)
-            asm volatile(
-                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                    su32(smem + W_OFF)),
-                "l"(w), "r"(W_BYTES), "r"(su32(bar))
-                : "memory");
+        if (j > 0)
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(su32(bar)), "r"(2u * PLANE_BYTES)
+                         : "memory");
 #pragma unroll
         for (int c = 0; c < 2; ++c)
             asm volatile(
@@ -177,14 +225,16 @@ __global__ void __launch_bounds__(128)
                 "l"(reinterpret_cast<uint64_t>(&tin)), "r"(8 * c), "r"(sl.x), "r"(sl.y), "r"(sl.z), "r"(su32(bar))
                 : "memory");
     };
-    if (tid == 0) {
-        load_halo(0);
-        if (J > 1) load_halo(1);
-    }
+    if (tid == 0) load_weights();
     const uint32_t tbase = tmem_base;
     float bz[CH];
 #pragma unroll
     for (int co = 0; co < CH; ++co) bz[co] = bias ? __ldg(bias + co) : 0.0f;
+    pdl_wait();
+    if (tid == 0) {
+        load_halo(0);
+        if (J > 1) load_halo(1);
+    }
     // epilogue of slab j: accumulator j & 1 -> bias, ReLU, gate -> output
     auto epilogue = [&](int j) {
         const int4 sl = slabs[blockIdx.x + j * G];
@@ -203,8 +253,8 @@ __global__ void __launch_bounds__(128)
             const size_t pc = pidx(b, x, y, z);
             uint4 gw[2] = {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
             if (gate) {  // the gate's 16 channels of this cell, two 16-byte loads
-                gw[0] = __ldg(reinterpret_cast<const uint4*>(gate + pc * CH));
-                gw[1] = __ldg(reinterpret_cast<const uint4*>(gate + pc * CH) + 1);
+                gw[0] = ld_u128(gate + pc * CH);
+                gw[1] = ld_u128(gate + pc * CH + 8);
             }
             const uint32_t* g32 = reinterpret_cast<const uint32_t*>(gw);
 #pragma unroll
@@ -328,11 +378,18 @@ static_assert((uint32_t)(((HZ - 1) * HY + (SL_Y - 2) + 2) * WG_ROW) + WG_ROW + 1
               "weight-gradient A operand reads past its buffer");
 static_assert((SL_Y - 2) * 256 + 256 + 128 + 128 <= (int)WG_B, "weight-gradient B operand reads past its buffer");
 
+// The three layers run in one launch (blockIdx.y: the layer), so one layer's tail fills with the next
+// one's CTAs: the three weight gradients depend on nothing but the back-propagated gradients.
+struct WgradArgs {
+    const __nv_bfloat16* dy[3];
+    const __nv_bfloat16* x[3];
+};
 __global__ void __launch_bounds__(128)
-    k_wgrad_tc(const __nv_bfloat16* __restrict__ dy, const __nv_bfloat16* __restrict__ x,
-               const int4* __restrict__ slabs, int n_slabs, Box b, float* __restrict__ part,
-               unsigned int* __restrict__ err)
+    k_wgrad_tc(WgradArgs in, const int4* __restrict__ slabs, int n_slabs, Box b, float* part_all, unsigned int* err)
 {
+    const __nv_bfloat16 *dy = in.dy[blockIdx.y], *x = in.x[blockIdx.y];
+    float* part = part_all + (size_t)blockIdx.y * WG_CTAS * (NW + CH);
+    pdl_trigger();
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) uint64_t bar_mma[2];
     __shared__ uint32_t tmem_base;
@@ -351,6 +408,7 @@ __global__ void __launch_bounds__(128)
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     __syncthreads();
+    pdl_wait();
     const uint32_t tbase = tmem_base;
     const uint32_t* x32 = reinterpret_cast<const uint32_t*>(x);
     const uint32_t* dy32 = reinterpret_cast<const uint32_t*>(dy);
@@ -377,8 +435,8 @@ __global__ void __launch_bounds__(128)
                 const int X = sl.x + ci8 + sx;
                 const bool ok = row_ok && X < b.px;
                 const size_t c8 = ok ? (((size_t)Z * b.py + Y) * b.px + X) * (CH / 2) : 0;
-                v[i][sx][0] = ok ? __ldg(x32 + c8 + cpw) : 0u;
-                v[i][sx][1] = ok ? __ldg(x32 + c8 + 4 + cpw) : 0u;
+                v[i][sx][0] = ok ? ld_u32(x32 + c8 + cpw) : 0u;
+                v[i][sx][1] = ok ? ld_u32(x32 + c8 + 4 + cpw) : 0u;
             }
         }
 #pragma unroll
@@ -387,7 +445,7 @@ __global__ void __launch_bounds__(128)
             const bool ok = X < b.nx && Y < b.ny;
             const size_t c8 = ok ? pidx(b, X, Y, sl.z) * (CH / 2) : 0;
 #pragma unroll
-            for (int g = 0; g < 2; ++g) u[i][g] = ok ? __ldg(dy32 + c8 + 4 * g + cpw) : 0u;
+            for (int g = 0; g < 2; ++g) u[i][g] = ok ? ld_u32(dy32 + c8 + 4 * g + cpw) : 0u;
         }
 #pragma unroll
         for (int i = 0; i < RW; ++i) {
@@ -503,21 +561,48 @@ __global__ void __launch_bounds__(128)
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tbase) : "memory");
 }
 
-// out[k] = sum over the n_part partial gradients of part[p][k] (weights and biases of one layer,
-// NW + CH values), in a fixed order: a CTA takes 32 consecutive k; its thread (c, k) adds the
-// partials p = c, c + 8, ... in increasing p, and the eight chunk sums are then added in
-// increasing c.
+// Position of weight (o, co, ci) in a layer's BF16 block, which is the convolution's shared-memory
+// layout (copied in as is): block o of 512 B holds the core matrices (co / 8, ci / 8) at 128-byte
+// steps, row co % 8 at 16-byte steps, ci % 8 within the row.
+__device__ __forceinline__ int w_layout(int o, int co, int ci)
+{
+    return o * 256 + (2 * (co >> 3) + (ci >> 3)) * 64 + (co & 7) * 8 + (ci & 7);
+}
+
+// BF16 forward weight r of layer l and its place in the data-gradient kernel
+// wt[o'][ci][co] = w[26 - o'][co][ci] (flipped offsets, transposed channels), both in w_layout.
+__device__ __forceinline__ void put_weight(int l, int r, float v, __nv_bfloat16* wb, __nv_bfloat16* wt)
+{
+    const int o = r / (CH * CH), co = (r / CH) % CH, ci = r % CH;
+    wb[l * NW + w_layout(o, co, ci)] = __float2bfloat16_rn(v);
+    wt[l * NW + w_layout(26 - o, ci, co)] = __float2bfloat16_rn(v);
+}
+
+// Adam's update of one parameter
+struct Adam {
+    float *p, *m, *v;
+    __nv_bfloat16 *wb, *wt;
+    float lr, b1, b2, eps, bc1, bc2;
+};
+
+// grad[l][k] = sum over the n_part partial gradients of layer l (weights and biases, NW + CH values), in
+// a fixed order: a CTA takes 32 consecutive k; its thread (c, k) adds the partials p = c, c + 8, ...
+// in increasing p, and the eight chunk sums are then added in increasing c.  In a training step the
+// thread that has the sum also takes the parameter's Adam step and writes its BF16 weights.
 constexpr int WR_K = 32, WR_C = 8;
+template <bool ADAM>
 __global__ void __launch_bounds__(WR_K * WR_C)
-    k_wgrad_reduce(const float* __restrict__ part, int n_part, float* __restrict__ out)
+    k_wgrad_reduce(const float* part_all, int n_part, float* grad, Adam ad)
 {
     __shared__ float cs[WR_C][WR_K];
-    const int kk = threadIdx.x % WR_K, c = threadIdx.x / WR_K;
+    const int kk = threadIdx.x % WR_K, c = threadIdx.x / WR_K, l = blockIdx.y;
     const int k = blockIdx.x * WR_K + kk;
+    const float* part = part_all + (size_t)l * WG_CTAS * (NW + CH);
+    pdl_wait();
     float s = 0.0f;
     if (k < NW + CH) {
 #pragma unroll 8
-        for (int p = c; p < n_part; p += WR_C) s += part[(size_t)p * (NW + CH) + k];
+        for (int p = c; p < n_part; p += WR_C) s += ld_f32(part + (size_t)p * (NW + CH) + k);
     }
     cs[c][kk] = s;
     __syncthreads();
@@ -525,7 +610,17 @@ __global__ void __launch_bounds__(WR_K * WR_C)
         float t = cs[0][kk];
 #pragma unroll
         for (int q = 1; q < WR_C; ++q) t += cs[q][kk];
-        out[k] = t;
+        const int i = l * (NW + CH) + k;
+        grad[i] = t;
+        if (ADAM) {
+            const float mi = ad.b1 * ad.m[i] + (1.0f - ad.b1) * t;
+            const float vi = ad.b2 * ad.v[i] + (1.0f - ad.b2) * t * t;
+            const float pi = ad.p[i] - ad.lr * (mi / ad.bc1) / (sqrtf(vi / ad.bc2) + ad.eps);
+            ad.m[i] = mi;
+            ad.v[i] = vi;
+            ad.p[i] = pi;
+            if (k < NW) put_weight(l, k, pi, ad.wb, ad.wt);
+        }
     }
 }
 
@@ -543,14 +638,32 @@ __device__ __forceinline__ bool slab_cell(const int4* slabs, const Box& b, int& 
     return x < b.nx && y < b.ny;
 }
 
-// Input features on the padded box: u / u_scale (3), (rho - 1) / rho_scale, fluid mask, zeros.
+// Input features on the padded box: u / u_scale (3), (rho - 1) / rho_scale, fluid mask, zeros.  On the way:
+// the caller's correction box is zeroed (zero, n_zero values; the slabs' cells are written later by the
+// last convolution), and the cells of a training step's output mask are counted.
 __global__ void __launch_bounds__(128) k_features(const float* __restrict__ rho, const float* __restrict__ u,
                                                   const uint8_t* __restrict__ mask, Box b, float inv_us, float inv_rs,
-                                                  __nv_bfloat16* __restrict__ x0, const int4* __restrict__ slabs)
+                                                  __nv_bfloat16* __restrict__ x0, const int4* __restrict__ slabs,
+                                                  float* __restrict__ zero, int64_t n_zero,
+                                                  const uint8_t* __restrict__ out_mask, unsigned long long* count)
 {
+    pdl_trigger();
     int x, y, z;
     int64_t c;
-    if (!slab_cell(slabs, b, x, y, z, c)) return;
+    const bool in = slab_cell(slabs, b, x, y, z, c);
+    if (zero) {
+        const int64_t t = (int64_t)blockIdx.x * 128 + threadIdx.x, stride = (int64_t)gridDim.x * 128;
+        if ((reinterpret_cast<uintptr_t>(zero) & 15u) == 0) {  // n_zero is a multiple of 4
+            for (int64_t k = t; k < n_zero / 4; k += stride) reinterpret_cast<float4*>(zero)[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        } else {
+            for (int64_t k = t; k < n_zero; k += stride) zero[k] = 0.0f;
+        }
+    }
+    if (count) {
+        const unsigned int ballot = __ballot_sync(0xffffffffu, in && out_mask[c] != 0);
+        if ((threadIdx.x & 31) == 0 && ballot) atomicAdd(count, (unsigned long long)__popc(ballot));
+    }
+    if (!in) return;
     const int64_t n = (int64_t)b.nx * b.ny * b.nz;
     const float fl = mask[c] ? 1.0f : 0.0f;
     __nv_bfloat16 v[CH];
@@ -568,24 +681,16 @@ __global__ void __launch_bounds__(128) k_features(const float* __restrict__ rho,
 
 // Loss = mean over fluid cells and components of (O - T)^2, T = (u_target - u) / du_scale;
 // dO = 2 (O - T) / N at fluid cells (BF16, padded, channels 0..2).
-__global__ void __launch_bounds__(128) k_count(const uint8_t* __restrict__ mask, Box b, const int4* __restrict__ slabs,
-                                               unsigned long long* __restrict__ count)
-{
-    int x, y, z;
-    int64_t c;
-    const bool in = slab_cell(slabs, b, x, y, z, c);
-    const unsigned int ballot = __ballot_sync(0xffffffffu, in && mask[c] != 0);
-    if ((threadIdx.x & 31) == 0 && ballot) atomicAdd(count, (unsigned long long)__popc(ballot));
-}
-
-__global__ void __launch_bounds__(128) k_loss(const float* __restrict__ o4, const float* __restrict__ u,
+__global__ void __launch_bounds__(128) k_loss(const float* o4, const float* __restrict__ u,
                                               const float* __restrict__ ut, const uint8_t* __restrict__ mask, Box b,
-                                              float inv_du, const unsigned long long* __restrict__ count,
-                                              __nv_bfloat16* __restrict__ dO, double* __restrict__ loss,
-                                              const int4* __restrict__ slabs)
+                                              float inv_du, const volatile unsigned long long* count,
+                                              __nv_bfloat16* dO, double* loss, const int4* __restrict__ slabs)
 {
     __shared__ double sh[4];
-    const float two_over_n = *count ? 2.0f / (3.0f * (float)*count) : 0.0f;
+    pdl_trigger();
+    pdl_wait();
+    const unsigned long long cells = *count;
+    const float two_over_n = cells ? 2.0f / (3.0f * (float)cells) : 0.0f;
     const int64_t n = (int64_t)b.nx * b.ny * b.nz;
     int x, y, z;
     int64_t c;
@@ -599,7 +704,7 @@ __global__ void __launch_bounds__(128) k_loss(const float* __restrict__ o4, cons
         for (int k = 0; k < 3; ++k) {
             float r = 0.0f;
             if (on) {
-                r = o4[c * 4 + k] - (ut[k * n + c] - u[k * n + c]) * inv_du;
+                r = ld_f32(o4 + c * 4 + k) - (ut[k * n + c] - u[k * n + c]) * inv_du;
                 part += (double)r * r;
             }
             d[k] = __float2bfloat16_rn(two_over_n * r);
@@ -611,67 +716,78 @@ __global__ void __launch_bounds__(128) k_loss(const float* __restrict__ o4, cons
     if (threadIdx.x == 0) atomicAdd(loss, (sh[0] + sh[1]) + (sh[2] + sh[3]));
 }
 
-// Position of weight (o, co, ci) in a layer's BF16 block, which is the convolution's shared-memory
-// layout (copied in as is): block o of 512 B holds the core matrices (co / 8, ci / 8) at 128-byte
-// steps, row co % 8 at 16-byte steps, ci % 8 within the row.
-__device__ __forceinline__ int w_layout(int o, int co, int ci)
-{
-    return o * 256 + (2 * (co >> 3) + (ci >> 3)) * 64 + (co & 7) * 8 + (ci & 7);
-}
-
-// BF16 forward weights and, for layers 2 and 3, the data-gradient kernels
-// wt[o'][ci][co] = w[26 - o'][co][ci] (flipped offsets, transposed channels), both in w_layout.
+// BF16 weights of all layers from the master parameters (at creation and after set_params)
 __global__ void k_prepare(const float* __restrict__ master, __nv_bfloat16* __restrict__ wb, __nv_bfloat16* __restrict__ wt)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= 3 * NW) return;
-    const int l = i / NW, r = i % NW;
-    const int o = r / (CH * CH), co = (r / CH) % CH, ci = r % CH;
-    const float v = master[l * (NW + CH) + r];
-    wb[l * NW + w_layout(o, co, ci)] = __float2bfloat16_rn(v);
-    wt[l * NW + w_layout(26 - o, ci, co)] = __float2bfloat16_rn(v);
+    put_weight(i / NW, i % NW, master[(i / NW) * (NW + CH) + i % NW], wb, wt);
 }
 
-__global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
-                       int n, float lr, float b1, float b2, float eps, float bc1, float bc2)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.0f - b1) * gi;
-    const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    p[i] -= lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
-}
-
-// coarse (X,Y,Z) = mean of rho and u over the fluid fine children (2X+a, 2Y+b, 2Z+c); 0 if none.
-__global__ void k_restrict(const float* __restrict__ frho, const float* __restrict__ fu, const uint8_t* __restrict__ fmask,
-                           int fnx, int fny, int fnz, float* __restrict__ crho, float* __restrict__ cu)
+// coarse (X,Y,Z) = mean of rho and u over the fluid fine children (2X+a, 2Y+b, 2Z+c); 0 if none.  A thread
+// takes W consecutive coarse cells of a row: with W = 4 the mask comes as four 8-byte words, most of
+// which are 0 (a vessel fills about 2% of its box), and the four planes go out as 16-byte stores, so
+// the kernel moves the mask and the coarse fields at memory speed; the fluid children are read one by
+// one, in the order of the sum (z, y, x), whatever W is.  W = 1: rows or arrays that the wide
+// accesses do not fit.  256^3 -> 128^3 vessel, cold: 26 us with one cell a thread.
+template <int W>
+__global__ void __launch_bounds__(256)
+    k_restrict(const float* __restrict__ frho, const float* __restrict__ fu, const uint8_t* __restrict__ fmask, int fnx,
+               int fny, int fnz, float* __restrict__ crho, float* __restrict__ cu)
 {
     const int cnx = fnx / 2, cny = fny / 2, cnz = fnz / 2;
     const int64_t cn = (int64_t)cnx * cny * cnz, fn = (int64_t)fnx * fny * fnz;
-    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * W;
     if (c >= cn) return;
-    const int X = (int)(c % cnx), Y = (int)((c / cnx) % cny), Z = (int)(c / ((int64_t)cnx * cny));
-    float sr = 0.f, su[3] = {0.f, 0.f, 0.f};
-    int k = 0;
-    for (int dz = 0; dz < 2; ++dz)
-        for (int dy = 0; dy < 2; ++dy)
-            for (int dx = 0; dx < 2; ++dx) {
-                const int64_t f = (int64_t)(2 * X + dx) + (int64_t)fnx * ((2 * Y + dy) + (int64_t)fny * (2 * Z + dz));
-                if (!fmask[f]) continue;
-                ++k;
-                sr += frho[f];
-                su[0] += fu[f];
-                su[1] += fu[fn + f];
-                su[2] += fu[2 * fn + f];
+    const uint32_t row = (uint32_t)(c / cnx);
+    const int X = (int)(c - (int64_t)row * cnx), Y = (int)(row % (uint32_t)cny), Z = (int)(row / (uint32_t)cny);
+    uint8_t m[4][2 * W];
+    int64_t at[4];
+    bool any = false;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        at[r] = 2 * X + (int64_t)fnx * ((2 * Y + (r & 1)) + (int64_t)fny * (2 * Z + (r >> 1)));
+        if constexpr (W == 4) {
+            const uint2 v = __ldg(reinterpret_cast<const uint2*>(fmask + at[r]));
+            memcpy(m[r], &v, 8);
+            any = any || (v.x | v.y);
+        } else {
+#pragma unroll
+            for (int x = 0; x < 2 * W; ++x) {
+                m[r][x] = fmask[at[r] + x];
+                any = any || m[r][x];
             }
-    const float inv = k ? 1.0f / (float)k : 0.0f;
-    crho[c] = sr * inv;
-    cu[c] = su[0] * inv;
-    cu[cn + c] = su[1] * inv;
-    cu[2 * cn + c] = su[2] * inv;
+        }
+    }
+    float o[4][W] = {};
+    if (any) {
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+            float s[4] = {0.f, 0.f, 0.f, 0.f};
+            int k = 0;
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int x = 0; x < 2; ++x) {
+                    if (!m[r][2 * w + x]) continue;
+                    const int64_t f = at[r] + 2 * w + x;
+                    ++k;
+                    s[0] += frho[f];
+                    s[1] += fu[f];
+                    s[2] += fu[fn + f];
+                    s[3] += fu[2 * fn + f];
+                }
+            const float inv = k ? 1.0f / (float)k : 0.0f;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) o[q][w] = s[q] * inv;
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        float* dst = q ? cu + (q - 1) * cn + c : crho + c;
+        if constexpr (W == 4) *reinterpret_cast<float4*>(dst) = make_float4(o[q][0], o[q][1], o[q][2], o[q][3]);
+        else dst[0] = o[q][0];
+    }
 }
 
 int blocks(int64_t n, int t) { return (int)((n + t - 1) / t); }
@@ -724,7 +840,15 @@ struct lbm_corrector {
     uint8_t* mask = nullptr;
     int4* slabs = nullptr;   // 8 x 16 x 1 slabs covering the 4^3 tiles with fluid, dilated by one tile
     int64_t n_slabs = 0;
-    unsigned int* err = nullptr;  // set by a conv CTA whose bounded wait gave up
+    // what a training pass reports, read back in one copy: the loss sum, the cells it runs over, and the
+    // error word set by a CTA whose bounded wait gave up
+    struct Report {
+        double loss;
+        unsigned long long count;
+        unsigned int err;
+    };
+    Report* report = nullptr;    // device
+    Report* h_report = nullptr;  // pinned
     cudaEvent_t ev = nullptr;     // orders the corrector's stream and a domain's stream (apply)
     CUtensorMap tmaps[5];         // halo maps of x0, y1, y2, dO, dy2 (the convolutions' inputs)
     const void* tmap_of[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
@@ -732,10 +856,8 @@ struct lbm_corrector {
     float* o4 = nullptr;
     float *rho = nullptr, *u = nullptr, *du = nullptr;  // staging on the coarse box
     float *master = nullptr, *grad = nullptr, *m = nullptr, *v = nullptr;
-    float* wpart = nullptr;  // [WG_CTAS][NW + CH] partial weight gradients of one layer
+    float* wpart = nullptr;  // [3][WG_CTAS][NW + CH] partial weight gradients of the layers
     __nv_bfloat16 *wb = nullptr, *wt = nullptr;
-    double* loss = nullptr;
-    unsigned long long* count = nullptr;
     int64_t adam_t = 0;
     int sms = 0;  // SMs of the device the corrector was created on
     uint64_t export_serial = 0;  // the domain whose zeros rho, u hold outside its fluid cells (0: none)
@@ -756,6 +878,8 @@ struct lbm_corrector {
     {
         if (ev) cudaEventDestroy(ev);
         ev = nullptr;
+        if (h_report) cudaFreeHost(h_report);
+        h_report = nullptr;
         for (void* p : owned) {
             if (release) release(p, ctx);
             else if (!alloc) cudaFree(p);
@@ -774,25 +898,32 @@ struct lbm_corrector {
         if (t == 5) return cudaErrorInvalidValue;
         const int grid = (int)std::min<int64_t>(n_slabs, (int64_t)sms * CONV_CTAS_PER_SM);
         auto k = mode == OUT_F32 ? k_conv_tc<OUT_F32> : mode == OUT_DU ? k_conv_tc<OUT_DU> : k_conv_tc<OUT_BF16>;
-        k<<<grid, 128, CONV_SMEM, stream>>>(tmaps[t], w, bias, relu, gate, out, slabs, (int)n_slabs, box, err, dua);
-        return cudaGetLastError();
+        return launch_pdl(k, dim3((unsigned)grid), 128, CONV_SMEM, stream, tmaps[t], w, bias, relu, gate, out, slabs,
+                          (int)n_slabs, box, &report->err, dua);
     }
-    // nonzero device error word (read after the stream has been synchronised)
-    bool device_error()
+    // enqueues the copy of the report, waits, and gives the mean loss; TIMEOUT if a CTA gave up
+    lbm_status finish(cudaError_t e, const char* what, double* loss)
     {
-        unsigned int h = 0;
-        if (cudaMemcpy(&h, err, sizeof(h), cudaMemcpyDeviceToHost) != cudaSuccess) return true;
-        if (h) cudaMemset(err, 0, sizeof(h));
-        return h != 0;
+        if (e == cudaSuccess) e = cudaMemcpyAsync(h_report, report, sizeof(Report), cudaMemcpyDeviceToHost, stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+        if (e != cudaSuccess) return nn_fail(LBM_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
+        if (h_report->err) {
+            cudaMemset(&report->err, 0, sizeof(unsigned int));
+            return nn_fail(LBM_ERR_TIMEOUT, "a convolution gave up waiting for its copies or MMAs");
+        }
+        *loss = h_report->count ? h_report->loss / (3.0 * (double)h_report->count) : 0.0;
+        return LBM_OK;
     }
     // the network on the slabs: O into o4 (du == nullptr), or, for an inference, the correction
-    // du = scale clamp(O[0:3]) at the cells of out_mask straight from the last layer
-    cudaError_t forward(const uint8_t* cmask, const float* r, const float* uu, float* du = nullptr,
-                        const uint8_t* out_mask = nullptr, float scale = 0.0f)
+    // du = scale clamp(O[0:3]) at the cells of out_mask straight from the last layer (zero_du: the rest
+    // of the caller's box is zeroed).  A training pass counts the cells of out_mask.
+    cudaError_t forward(const uint8_t* cmask, const float* r, const float* uu, float* du, const uint8_t* out_mask,
+                        float scale, bool zero_du)
     {
-        if (n_slabs == 0) return cudaSuccess;
+        if (n_slabs == 0) return zero_du ? cudaMemsetAsync(du, 0, sizeof(float) * 3 * n_cells, stream) : cudaSuccess;
         k_features<<<(unsigned)n_slabs, 128, 0, stream>>>(r, uu, cmask ? cmask : mask, box, 1.0f / u_scale,
-                                                          1.0f / rho_scale, x0, slabs);
+                                                          1.0f / rho_scale, x0, slabs, zero_du ? du : nullptr,
+                                                          3 * n_cells, out_mask, du ? nullptr : &report->count);
         cudaError_t e = cudaGetLastError();
         if (e == cudaSuccess) e = conv(x0, wb, bmaster(0), 1, nullptr, y1, OUT_BF16);
         if (e == cudaSuccess) e = conv(y1, wb + NW, bmaster(1), 1, nullptr, y2, OUT_BF16);
@@ -800,31 +931,30 @@ struct lbm_corrector {
         if (e == cudaSuccess && du) e = conv(y2, wb + 2 * NW, bmaster(2), 0, nullptr, du, OUT_DU, DuArgs{out_mask, scale, clip});
         return e;
     }
-    // loss and gradients into `grad` (FP32, parameter layout), loss into `loss`
-    cudaError_t backward(const uint8_t* mk, const float* uu, const float* ut)
+    // forward pass, loss and gradients into `grad` (FP32, parameter layout), the report, and, with `ad`, an
+    // Adam step.  Convolutions first, then the three weight gradients in one launch and their sums in
+    // another: 9 kernels and one clear, against 17 and 3 with a launch per layer and per elementwise step.
+    cudaError_t train(const uint8_t* cmask, const uint8_t* mk, const float* r, const float* uu, const float* ut, const Adam* ad)
     {
-        cudaError_t e = cudaMemsetAsync(grad, 0, sizeof(float) * NP, stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(loss, 0, sizeof(double), stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(count, 0, sizeof(unsigned long long), stream);
+        cudaError_t e = cudaMemsetAsync(report, 0, offsetof(Report, err), stream);
+        if (e == cudaSuccess) e = forward(cmask, r, uu, nullptr, mk, 0.0f, false);
         if (e != cudaSuccess) return e;
-        if (n_slabs) {
-            k_count<<<(unsigned)n_slabs, 128, 0, stream>>>(mk, box, slabs, count);
-            k_loss<<<(unsigned)n_slabs, 128, 0, stream>>>(o4, uu, ut, mk, box, 1.0f / du_scale, count, dO, loss, slabs);
+        if (n_slabs == 0) {  // no cell: zero gradients, and Adam's moments decay
+            e = cudaMemsetAsync(wpart, 0, sizeof(float) * 3 * (size_t)WG_CTAS * (NW + CH), stream);
+        } else {
+            e = launch_pdl(k_loss, dim3((unsigned)n_slabs), 128, 0, stream, o4, uu, ut, mk, box, 1.0f / du_scale, &report->count,
+                           dO, &report->loss, slabs);
+            // dz2 = W3^T dO gated by y2 > 0, dz1 = W2^T dz2 gated by y1 > 0
+            if (e == cudaSuccess) e = conv(dO, wt + 2 * NW, nullptr, 0, y2, dy2, OUT_BF16);
+            if (e == cudaSuccess) e = conv(dy2, wt + NW, nullptr, 0, y1, dy, OUT_BF16);
         }
-        e = cudaGetLastError();
         const int wg = (int)std::min<int64_t>(std::max<int64_t>(n_slabs, 1), WG_CTAS);
-        // weight gradient of one layer: per-CTA partials, then their sum in a fixed order
-        auto wgrad = [&](const __nv_bfloat16* g, const __nv_bfloat16* xin, float* out) {
-            if (!n_slabs) return cudaSuccess;
-            k_wgrad_tc<<<wg, 128, WG_SMEM, stream>>>(g, xin, slabs, (int)n_slabs, box, wpart, err);
-            k_wgrad_reduce<<<blocks(NW + CH, WR_K), WR_K * WR_C, 0, stream>>>(wpart, wg, out);
-            return cudaGetLastError();
-        };
-        if (e == cudaSuccess) e = wgrad(dO, y2, grad + 2 * (NW + CH));
-        if (e == cudaSuccess) e = conv(dO, wt + 2 * NW, nullptr, 0, y2, dy2, OUT_BF16);  // dz2 = W3^T dO, gated by y2 > 0
-        if (e == cudaSuccess) e = wgrad(dy2, y1, grad + (NW + CH));
-        if (e == cudaSuccess) e = conv(dy2, wt + NW, nullptr, 0, y1, dy, OUT_BF16);  // dz1 = W2^T dz2, gated by y1 > 0
-        if (e == cudaSuccess) e = wgrad(dy, x0, grad);
+        if (e == cudaSuccess && n_slabs)
+            e = launch_pdl(k_wgrad_tc, dim3((unsigned)wg, 3), 128, WG_SMEM, stream, WgradArgs{{dy, dy2, dO}, {x0, y1, y2}}, slabs,
+                           (int)n_slabs, box, wpart, &report->err);
+        if (e == cudaSuccess)
+            e = launch_pdl(ad ? k_wgrad_reduce<true> : k_wgrad_reduce<false>, dim3((unsigned)blocks(NW + CH, WR_K), 3),
+                           WR_K * WR_C, 0, stream, wpart, wg, grad, ad ? *ad : Adam{});
         return e;
     }
     cudaError_t prepare()
@@ -911,7 +1041,7 @@ lbm_status lbm_corrector_create(const uint8_t* mask, int32_t nx, int32_t ny, int
     };
     K->mask = static_cast<uint8_t*>(D(cells));
     K->slabs = static_cast<int4*>(D(sizeof(int4) * std::max<size_t>(sv.size(), 1)));
-    K->err = static_cast<unsigned int*>(D(sizeof(unsigned int)));
+    K->report = static_cast<lbm_corrector::Report*>(D(sizeof(lbm_corrector::Report)));
     K->x0 = static_cast<__nv_bfloat16*>(D(act));
     K->y1 = static_cast<__nv_bfloat16*>(D(act));
     K->y2 = static_cast<__nv_bfloat16*>(D(act));
@@ -926,11 +1056,9 @@ lbm_status lbm_corrector_create(const uint8_t* mask, int32_t nx, int32_t ny, int
     K->grad = static_cast<float*>(D(sizeof(float) * NP));
     K->m = static_cast<float*>(D(sizeof(float) * NP));
     K->v = static_cast<float*>(D(sizeof(float) * NP));
-    K->wpart = static_cast<float*>(D(sizeof(float) * (size_t)WG_CTAS * (NW + CH)));
+    K->wpart = static_cast<float*>(D(sizeof(float) * 3 * (size_t)WG_CTAS * (NW + CH)));
     K->wb = static_cast<__nv_bfloat16*>(D(sizeof(__nv_bfloat16) * 3 * NW));
     K->wt = static_cast<__nv_bfloat16*>(D(sizeof(__nv_bfloat16) * 3 * NW));
-    K->loss = static_cast<double*>(D(sizeof(double)));
-    K->count = static_cast<unsigned long long*>(D(sizeof(unsigned long long)));
     if (!ok) {
         K->release_all();
         delete K;
@@ -939,7 +1067,8 @@ lbm_status lbm_corrector_create(const uint8_t* mask, int32_t nx, int32_t ny, int
     cudaError_t e = cudaMemcpyAsync(K->mask, mask, cells, cudaMemcpyHostToDevice, K->stream);
     if (e == cudaSuccess && !sv.empty())
         e = cudaMemcpyAsync(K->slabs, sv.data(), sizeof(int4) * sv.size(), cudaMemcpyHostToDevice, K->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(K->err, 0, sizeof(unsigned int), K->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(K->report, 0, sizeof(lbm_corrector::Report), K->stream);
+    if (e == cudaSuccess) e = cudaMallocHost((void**)&K->h_report, sizeof(lbm_corrector::Report));
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&K->ev, cudaEventDisableTiming);
     {  // the convolutions' grid and their shared-memory sizes, once
         int dev = 0;
@@ -1005,8 +1134,7 @@ lbm_status lbm_corrector_forward(lbm_corrector* K, const uint8_t* mask, const ui
     if (!K || !rho || !u || !du) return nn_fail(LBM_ERR_INVALID_ARG, "NULL argument");
     const uint8_t* om = out_mask ? out_mask : (mask ? mask : K->mask);
     // the slabs write their cells; the rest of the caller's box is zero
-    cudaError_t e = cudaMemsetAsync(du, 0, sizeof(float) * 3 * K->n_cells, K->stream);
-    if (e == cudaSuccess) e = K->forward(mask, rho, u, du, om, K->du_scale);
+    cudaError_t e = K->forward(mask, rho, u, du, om, K->du_scale, true);
     if (e != cudaSuccess) return nn_fail(LBM_ERR_CUDA, std::string("corrector forward: ") + cudaGetErrorString(e));
     return LBM_OK;
 }
@@ -1016,18 +1144,9 @@ lbm_status lbm_corrector_gradients(lbm_corrector* K, const uint8_t* mask, const 
 {
     NvtxRange nvtx_range("lbm_corrector_gradients");
     if (!K || !rho || !u || !u_target || !grad || !loss) return nn_fail(LBM_ERR_INVALID_ARG, "NULL argument");
-    cudaError_t e = K->forward(mask, rho, u);
-    if (e == cudaSuccess) e = K->backward(out_mask ? out_mask : (mask ? mask : K->mask), u, u_target);
+    cudaError_t e = K->train(mask, out_mask ? out_mask : (mask ? mask : K->mask), rho, u, u_target, nullptr);
     if (e == cudaSuccess) e = cudaMemcpyAsync(grad, K->grad, sizeof(float) * NP, cudaMemcpyDeviceToHost, K->stream);
-    double l = 0.0;
-    unsigned long long cnt = 0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&l, K->loss, sizeof(double), cudaMemcpyDeviceToHost, K->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&cnt, K->count, sizeof(cnt), cudaMemcpyDeviceToHost, K->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(K->stream);
-    if (e != cudaSuccess) return nn_fail(LBM_ERR_CUDA, std::string("corrector gradients: ") + cudaGetErrorString(e));
-    if (K->device_error()) return nn_fail(LBM_ERR_TIMEOUT, "a convolution gave up waiting for its copies or MMAs");
-    *loss = cnt ? l / (3.0 * (double)cnt) : 0.0;
-    return LBM_OK;
+    return K->finish(e, "corrector gradients", loss);
 }
 
 lbm_status lbm_corrector_train_step(lbm_corrector* K, const uint8_t* mask, const uint8_t* out_mask, const float* rho,
@@ -1036,26 +1155,13 @@ lbm_status lbm_corrector_train_step(lbm_corrector* K, const uint8_t* mask, const
     NvtxRange nvtx_range("lbm_corrector_train_step");
     if (!K || !rho || !u || !u_target) return nn_fail(LBM_ERR_INVALID_ARG, "NULL argument");
     if (!(lr > 0.0)) return nn_fail(LBM_ERR_INVALID_ARG, "lr must be > 0");
-    cudaError_t e = K->forward(mask, rho, u);
-    if (e == cudaSuccess) e = K->backward(out_mask ? out_mask : (mask ? mask : K->mask), u, u_target);
     K->adam_t += 1;
     const float b1 = 0.9f, b2 = 0.999f;
     const float bc1 = 1.0f - std::pow(b1, (float)K->adam_t), bc2 = 1.0f - std::pow(b2, (float)K->adam_t);
-    if (e == cudaSuccess) {
-        k_adam<<<blocks(NP, 256), 256, 0, K->stream>>>(K->master, K->grad, K->m, K->v, NP, (float)lr, b1, b2, 1e-8f,
-                                                       bc1, bc2);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = K->prepare();
-    double l = 0.0;
-    unsigned long long cnt = 0;
-    if (e == cudaSuccess && loss) e = cudaMemcpyAsync(&l, K->loss, sizeof(double), cudaMemcpyDeviceToHost, K->stream);
-    if (e == cudaSuccess && loss) e = cudaMemcpyAsync(&cnt, K->count, sizeof(cnt), cudaMemcpyDeviceToHost, K->stream);
-    if (e == cudaSuccess && loss) e = cudaStreamSynchronize(K->stream);
+    const Adam ad{K->master, K->m, K->v, K->wb, K->wt, (float)lr, b1, b2, 1e-8f, bc1, bc2};
+    cudaError_t e = K->train(mask, out_mask ? out_mask : (mask ? mask : K->mask), rho, u, u_target, &ad);
+    if (loss) return K->finish(e, "corrector train step", loss);
     if (e != cudaSuccess) return nn_fail(LBM_ERR_CUDA, std::string("corrector train step: ") + cudaGetErrorString(e));
-    if (loss && K->device_error())
-        return nn_fail(LBM_ERR_TIMEOUT, "a convolution gave up waiting for its copies or MMAs");
-    if (loss) *loss = cnt ? l / (3.0 * (double)cnt) : 0.0;
     return LBM_OK;
 }
 
@@ -1083,7 +1189,7 @@ lbm_status lbm_corrector_apply(lbm_corrector* K, lbm_domain* dom, const uint8_t*
     }
     const uint8_t* om = out_mask ? out_mask : (mask ? mask : K->mask);
     // cells outside the slabs keep the zero of set-up
-    if (e == cudaSuccess) e = K->forward(mask, K->rho, K->u, K->du, om, (float)(K->du_scale * gain));
+    if (e == cudaSuccess) e = K->forward(mask, K->rho, K->u, K->du, om, (float)(K->du_scale * gain), false);
     if (e == cudaSuccess && da.stream != K->stream) {
         e = cudaEventRecord(K->ev, K->stream);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(da.stream, K->ev, 0);
@@ -1110,8 +1216,14 @@ lbm_status lbm_restrict(const float* fine_rho, const float* fine_u, const uint8_
     if (fnx <= 0 || fny <= 0 || fnz <= 0 || fnx % 2 || fny % 2 || fnz % 2)
         return nn_fail(LBM_ERR_INVALID_ARG, "fine extents must be positive and even");
     const int64_t cn = (int64_t)(fnx / 2) * (fny / 2) * (fnz / 2);
-    k_restrict<<<blocks(cn, 256), 256, 0, static_cast<cudaStream_t>(cuda_stream)>>>(fine_rho, fine_u, fine_mask, fnx, fny,
-                                                                                     fnz, coarse_rho, coarse_u);
+    const cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    // rows of whole groups of four coarse cells, and arrays on the boundaries of the wide accesses
+    const bool wide = fnx % 8 == 0 && (reinterpret_cast<uintptr_t>(fine_mask) & 7u) == 0 &&
+                      ((reinterpret_cast<uintptr_t>(coarse_rho) | reinterpret_cast<uintptr_t>(coarse_u)) & 15u) == 0;
+    if (wide)
+        k_restrict<4><<<blocks(cn / 4, 256), 256, 0, st>>>(fine_rho, fine_u, fine_mask, fnx, fny, fnz, coarse_rho, coarse_u);
+    else
+        k_restrict<1><<<blocks(cn, 256), 256, 0, st>>>(fine_rho, fine_u, fine_mask, fnx, fny, fnz, coarse_rho, coarse_u);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return nn_fail(LBM_ERR_CUDA, std::string("restrict: ") + cudaGetErrorString(e));
     return LBM_OK;
