@@ -998,6 +998,15 @@ __device__ __forceinline__ void gather(const DomainView& v, const void* src, uin
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Rounds of links a warp holds in registers: six cover every run of the vessels, so no warp of a small
+// domain, whose step is as long as its slowest warp, waits for the reloading loop (25 k cells: 6.5 -> 5.3 us,
+// 150 k: 10.3 -> 9.5 us against three); on a large domain the warps hide one another's latency and the fewer
+// registers win (2.7 M cells, 45 k bricks: 124 us with three, 129 us with six; 11 k bricks: 26.0 and 26.9 us).
+constexpr int LINK_ROUNDS = 6, LINK_ROUNDS_LARGE = 3;
+// Bricks from which a domain counts as large here and in the default launch configuration: several waves of
+// CTAs, so that throughput counts and not the slowest warp.
+constexpr int64_t LARGE_BRICKS = 8192;
+
 // Bouzidi links of a warp's cells, shared out among its lanes: the links of a half-brick are one run of the
 // packed list, so a lane takes entry k0 + lane, + 32, ...: code and coefficient (coalesced, before
 // pdl_wait: they never change), f*_a of the q >= 1/2 links (coalesced from the side buffer).  The cells'
@@ -1007,24 +1016,34 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // values there, from which the lanes keep f*_a.  About 60 instructions a cell and 25 per 32 links, and one
 // memory latency, against 27 directions x (test, position, two predicated loads, mix) in three groups
 // of a latency each when every cell handled its own links; a boundary half-brick has 50 to 100 links.
-// Per step, before -> after: 256^3 aneurysm FP32 11.9 -> 11.0 us, 2.7 M cell Bouzidi pipe 133.5 -> 128.8 us,
-// 25 k cell TRT aneurysm 7.7 -> 6.6 us, batch of 8 FP16 aneurysms 19.3 -> 17.1 us (with the closure by
-// face above).
-template <int ST, int SCHEME, int STRIDE>
+// Per step, each cell by itself -> this: 256^3 aneurysm FP32 11.9 -> 9.9 us, 2.7 M cell Bouzidi pipe 133.5 ->
+// 122.6 us, 25 k cell TRT aneurysm 7.7 -> 5.3 us, batch of 8 FP16 aneurysms 19.3 -> 15.6 us (with the closure
+// by face above and the register budget of large domains).
+// R: rounds of 32 links held in registers, in groups of three whose exchange reads come before their writes
+// (one shared-memory latency a group); longer runs reload their codes, a memory latency each.  On the synthetic
+// vessels a half-brick with links has 70 on average, up to 183, a fifth of them over 96 (LINK_ROUNDS).
+template <int ST, int SCHEME, int STRIDE, int R>
 struct BouzidiLinks {
-    static constexpr int R = 3;  // rounds of 32 links held in registers; longer runs reload
+    static constexpr int G = 3;
+    static_assert(R % G == 0, "whole groups");
     uint32_t k0, k1, lane;
-    uint32_t code[R];
+    uint32_t code[(R + 1) / 2];  // two 16-bit codes each
     float coef[R], fa[R];
 
     __device__ __forceinline__ bool any() const { return k0 < k1; }
-    __device__ __forceinline__ void load(const DomainView& v, uint32_t k, uint32_t& c, float& b) const
+    __device__ __forceinline__ bool round(int r) const { return k0 + 32u * r < k1; }  // the same in every lane
+    __device__ __forceinline__ uint32_t code_of(int r) const { return (code[r / 2] >> (16 * (r & 1))) & 0xffffu; }
+    __device__ __forceinline__ uint32_t load_code(const DomainView& v, uint32_t k) const
     {
-        const bool in = k < k1 && LBM_IN_RANGE(k, v.n_bq, 5);
-        c = in ? (uint32_t)__ldg(v.blink + k) : 0u;
-        b = in ? __ldg(v.bq + k) : 0.0f;
+        return k < k1 && LBM_IN_RANGE(k, v.n_bq, 5) ? (uint32_t)__ldg(v.blink + k) : 0u;
     }
-    __device__ __forceinline__ void prefetch(const DomainView& v, uint32_t half_brick, uint32_t lane_)
+    __device__ __forceinline__ float load_coef(const DomainView& v, uint32_t k) const
+    {
+        return k < k1 && LBM_IN_RANGE(k, v.n_bq, 5) ? __ldg(v.bq + k) : 0.0f;
+    }
+    // the run's bounds, then (prefetch) its codes and coefficients: the bounds are loaded beside the warp's other
+    // tables, so that the branch on them does not hold those back
+    __device__ __forceinline__ void begin(const DomainView& v, uint32_t half_brick, uint32_t lane_)
     {
         lane = lane_;
         k0 = k1 = 0u;
@@ -1032,8 +1051,24 @@ struct BouzidiLinks {
             k0 = (uint32_t)__ldg(v.bstart + half_brick);
             k1 = (uint32_t)__ldg(v.bstart + half_brick + 1);
         }
+    }
+    __device__ __forceinline__ void prefetch(const DomainView& v)
+    {
 #pragma unroll
-        for (int r = 0; r < R; ++r) load(v, k0 + 32u * r + lane, code[r], coef[r]);
+        for (int r = 0; r < R; ++r) coef[r] = 0.0f;
+#pragma unroll
+        for (int r = 0; r < (R + 1) / 2; ++r) code[r] = 0u;
+#pragma unroll
+        for (int r = 0; r < R; r += 2) {
+            if (!round(r)) break;  // the warps without links skip all of it
+            const uint32_t k = k0 + 32u * r + lane;
+            code[r / 2] = load_code(v, k);
+            coef[r] = load_coef(v, k);
+            if (r + 1 < R) {
+                code[r / 2] |= load_code(v, k + 32u) << 16;
+                coef[r + 1] = load_coef(v, k + 32u);
+            }
+        }
     }
     // f*_a of a q >= 1/2 link, as stored
     __device__ __forceinline__ float load_fa(const DomainView& v, const void* src, uint32_t slot0, uint32_t k, uint32_t c,
@@ -1047,31 +1082,50 @@ struct BouzidiLinks {
     __device__ __forceinline__ void issue(const DomainView& v, const void* src, uint32_t slot0)
     {
 #pragma unroll
-        for (int r = 0; r < R; ++r) fa[r] = load_fa(v, src, slot0, k0 + 32u * r + lane, code[r], coef[r]);
-    }
-    __device__ __forceinline__ void mix(uint32_t c, float b, float other, float* sm) const
-    {
-        if (b == 0.0f) return;  // past the end, or halfway bounce-back
-        const uint32_t cell = c & 31u, dir = (c >> 5) & 31u;
-        float& f = sm[dir * STRIDE + cell];
-        if (b < 0.0f) {
-            // 16-bit storages: w = w_of(13) 4^-nnz, the same float as w_of of the direction
-            const float w = Store<ST>::SCALED ? __int_as_float(__float_as_int(w_of(13)) - (int)(((c >> 11) & 3u) << 24)) : 1.0f;
-            f = wall_high(-b, f, Store<ST>::SCALED ? __fmul_rn(w, other) : other);
-        } else if (!(c & (1u << 10))) {
-            f = wall_low(b, f, sm[(Q - 1 - dir) * STRIDE + cell]);
+        for (int r = 0; r < R; ++r) {
+            if (r % 2 == 0 && !round(r)) break;
+            fa[r] = load_fa(v, src, slot0, k0 + 32u * r + lane, code_of(r), coef[r]);
         }
+    }
+    static __device__ __forceinline__ uint32_t at(uint32_t c) { return ((c >> 5) & 31u) * STRIDE + (c & 31u); }
+    // whether the link changes its value (past the end, halfway bounce-back, walls on both sides: no)
+    static __device__ __forceinline__ bool active(uint32_t c, float b) { return b < 0.0f || (b > 0.0f && !(c & (1u << 10))); }
+    static __device__ __forceinline__ float mix(uint32_t c, float b, float f, float other)
+    {
+        if (b > 0.0f) return wall_low(b, f, other);
+        // 16-bit storages: w = w_of(13) 4^-nnz, the same float as w_of of the direction
+        const float w = Store<ST>::SCALED ? __int_as_float(__float_as_int(w_of(13)) - (int)(((c >> 11) & 3u) << 24)) : 1.0f;
+        return wall_high(-b, f, Store<ST>::SCALED ? __fmul_rn(w, other) : other);
+    }
+    static __device__ __forceinline__ float other_value(uint32_t c, float b, float fa_, const float* sm)
+    {
+        return b < 0.0f ? fa_ : sm[(Q - 1 - ((c >> 5) & 31u)) * STRIDE + (c & 31u)];
     }
     __device__ __forceinline__ void apply(const DomainView& v, const void* src, uint32_t slot0, float* sm)
     {
         __syncwarp();
 #pragma unroll
-        for (int r = 0; r < R; ++r) mix(code[r], coef[r], fa[r], sm);
+        for (int g = 0; g < R; g += G) {
+            if (!round(g)) break;
+            float f[G], o[G];
+#pragma unroll
+            for (int r = 0; r < G; ++r) {
+                const uint32_t c = code_of(g + r);
+                if (active(c, coef[g + r])) {
+                    f[r] = sm[at(c)];
+                    o[r] = other_value(c, coef[g + r], fa[g + r], sm);
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < G; ++r) {
+                const uint32_t c = code_of(g + r);
+                if (active(c, coef[g + r])) sm[at(c)] = mix(c, coef[g + r], f[r], o[r]);
+            }
+        }
         for (uint32_t k = k0 + 32u * R + lane; k < k1; k += 32u) {
-            uint32_t c;
-            float b;
-            load(v, k, c, b);
-            mix(c, b, load_fa(v, src, slot0, k, c, b), sm);
+            const uint32_t c = load_code(v, k);
+            const float b = load_coef(v, k);
+            if (active(c, b)) sm[at(c)] = mix(c, b, sm[at(c)], other_value(c, b, load_fa(v, src, slot0, k, c, b), sm));
         }
         __syncwarp();
     }
@@ -1079,22 +1133,26 @@ struct BouzidiLinks {
     {
         __syncwarp();
 #pragma unroll
-        for (int r = 0; r < R; ++r)
-            if (coef[r] < 0.0f) Store<ST>::store_h(v.side, k0 + 32u * r + lane, sm[((code[r] >> 5) & 31u) * STRIDE + (code[r] & 31u)]);
-        for (uint32_t k = k0 + 32u * R + lane; k < k1; k += 32u) {
-            uint32_t c;
-            float b;
-            load(v, k, c, b);
-            if (b < 0.0f) Store<ST>::store_h(v.side, k, sm[((c >> 5) & 31u) * STRIDE + (c & 31u)]);
+        for (int g = 0; g < R; g += G) {
+            if (!round(g)) break;
+            float f[G];
+#pragma unroll
+            for (int r = 0; r < G; ++r)
+                if (coef[g + r] < 0.0f) f[r] = sm[at(code_of(g + r))];
+#pragma unroll
+            for (int r = 0; r < G; ++r)
+                if (coef[g + r] < 0.0f) Store<ST>::store_h(v.side, k0 + 32u * (g + r) + lane, f[r]);
         }
+        for (uint32_t k = k0 + 32u * R + lane; k < k1; k += 32u)
+            if (load_coef(v, k) < 0.0f) Store<ST>::store_h(v.side, k, sm[at(load_code(v, k))]);
     }
 };
 
 // One fused update of the cell at `slot` (a lane of a warp that covers half of one brick; all
 // 32 lanes must call it together: the neighbour row goes round by shuffle, the Bouzidi links are shared
-// out).  PDL: the kernel is launched as a programmatic dependent (not the persistent batch).  LINKS: the
-// domain may have Bouzidi cells; sm is then the warp's [27][32] exchange area.
-template <int ST, int SCHEME, int COLL, int PC = -1, bool PDL = true, bool LINKS = true>
+// out).  PDL: the kernel is launched as a programmatic dependent (not the persistent batch).  LINKS: the rounds
+// of BouzidiLinks, 0 for a domain without Bouzidi cells; else sm is the warp's [27][32] exchange area.
+template <int ST, int SCHEME, int COLL, int PC = -1, bool PDL = true, int LINKS = LINK_ROUNDS>
 __device__ __forceinline__ void step_cell(const DomainView& v, const void* src, void* dst, const LevelArgs& a,
                                           uint32_t slot, uint32_t lane, float* sm)
 {
@@ -1105,8 +1163,8 @@ __device__ __forceinline__ void step_cell(const DomainView& v, const void* src, 
     // the cell's record, loaded beside its word rather than after it: an open cell then waits for one
     // memory latency fewer (4 bytes per slot of traffic)
     const int32_t auxv = __ldg(v.aux + slot);
-    BouzidiLinks<ST, SCHEME, 32> links;
-    if (LINKS) links.prefetch(v, slot / 32u, lane);
+    BouzidiLinks<ST, SCHEME, 32, LINKS ? LINKS : 3> links;
+    if (LINKS) links.begin(v, slot / 32u, lane);
     const bool fluid = (word & WORD_FLUID) != 0u;
     const bool bouzidi = ((word >> WORD_KIND_SHIFT) & 3u) == KIND_BOUZIDI;
     const uint32_t wm = word & WORD_WALL_MASK;
@@ -1119,10 +1177,12 @@ __device__ __forceinline__ void step_cell(const DomainView& v, const void* src, 
         const int32_t row = __ldg(v.nb8 + brick * 8u + (lane & 7u));
         corner_slots_shfl(row, slot, cs);
         const bool clean = PC >= 0 && __all_sync(0xffffffffu, wm == 0u);
+        if (LINKS) links.prefetch(v);
         if (PDL) pdl_wait();
         if (fluid) fetch_et<ST, true, PC>(dst, n, cs, wm, a.parity, d, clean);
     } else {
         const int32_t row = __ldg(v.nbr + brick * (uint32_t)Q + (lane < (uint32_t)Q ? lane : 0u));
+        if (LINKS) links.prefetch(v);
         if (PDL) pdl_wait();
         fetch_ab_shfl<ST>(src, n, row, slot, wm, fluid, d);
     }
@@ -1156,7 +1216,7 @@ __device__ __forceinline__ void step_cell(const DomainView& v, const void* src, 
     }
 }
 
-template <int ST, int SCHEME, int BRICKS, int MINB, int COLL, int PC = -1, bool LINKS = true>
+template <int ST, int SCHEME, int BRICKS, int MINB, int COLL, int PC = -1, int LINKS = LINK_ROUNDS>
 __global__ void __launch_bounds__(BRICKS * BRICK_CELLS, MINB)
     k_step(DomainView v, const void* src, void* dst, LevelArgs a)
 {
@@ -1731,14 +1791,15 @@ cudaError_t launch_step_t(const DomainView& v, const void* src, void* dst, const
         constexpr int C = decltype(c)::value;
         constexpr int T = BRICKS * BRICK_CELLS;
         // the default rates: a domain without Bouzidi cells runs without the link code and its exchange area
-        // (64x64x256 pipe FP16 19.9 us a step, 20.8 us with them), and the twist has one kernel
-        // per parity (constant plane indices)
-        if constexpr (SCHEME == LBM_SCHEME_ESOTERIC && C == COLL_CHM_FAST) {
-            auto k = v.bstart ? (a.parity ? k_step<ST, SCHEME, BRICKS, MINB, C, 1> : k_step<ST, SCHEME, BRICKS, MINB, C, 0>)
-                              : (a.parity ? k_step<ST, SCHEME, BRICKS, MINB, C, 1, false> : k_step<ST, SCHEME, BRICKS, MINB, C, 0, false>);
-            return launch_pdl(k, grid, T, 0, s, v, src, dst, a);
-        } else if constexpr (C == COLL_CHM_FAST) {
-            auto k = v.bstart ? k_step<ST, SCHEME, BRICKS, MINB, C> : k_step<ST, SCHEME, BRICKS, MINB, C, -1, false>;
+        // (64x64x256 pipe FP16 19.5 us a step, 20.8 us with them), a large one with fewer rounds, and the
+        // twist has one kernel per parity (constant plane indices)
+        if constexpr (C == COLL_CHM_FAST) {
+            constexpr int P0 = SCHEME == LBM_SCHEME_ESOTERIC ? 0 : -1, P1 = SCHEME == LBM_SCHEME_ESOTERIC ? 1 : -1;
+            constexpr int L = LINK_ROUNDS, LL = LINK_ROUNDS_LARGE;
+            const bool large = v.n_bricks > LARGE_BRICKS;
+            auto k = !v.bstart ? (a.parity ? k_step<ST, SCHEME, BRICKS, MINB, C, P1, 0> : k_step<ST, SCHEME, BRICKS, MINB, C, P0, 0>)
+                     : large   ? (a.parity ? k_step<ST, SCHEME, BRICKS, MINB, C, P1, LL> : k_step<ST, SCHEME, BRICKS, MINB, C, P0, LL>)
+                               : (a.parity ? k_step<ST, SCHEME, BRICKS, MINB, C, P1, L> : k_step<ST, SCHEME, BRICKS, MINB, C, P0, L>);
             return launch_pdl(k, grid, T, 0, s, v, src, dst, a);
         } else {
             return launch_pdl(k_step<ST, SCHEME, BRICKS, MINB, C>, grid, T, 0, s, v, src, dst, a);
@@ -1790,7 +1851,11 @@ cudaError_t launch_step_scheme(int config, const DomainView& v, const void* src,
     switch (config) {
     case 0: return launch_step_t<ST, SCHEME, 4, 3>(v, src, dst, a, s);
     case 1: return launch_step_t<ST, SCHEME, 2, 7>(v, src, dst, a, s);
-    case 2: return launch_step_t<ST, SCHEME, 2, 6>(v, src, dst, a, s);
+    // the default: 6 CTAs per SM, 8 on large domains, which the memory system bounds and more loads in flight
+    // help (2.7 M cells FP32 124.6 -> 117.1 us, FP16 105.1 -> 88.7 us; 150 k cells 9.3 -> 9.5 us the other way)
+    case 2:
+        return v.n_bricks > LARGE_BRICKS ? launch_step_t<ST, SCHEME, 2, 8>(v, src, dst, a, s)
+                                         : launch_step_t<ST, SCHEME, 2, 6>(v, src, dst, a, s);
     case 3: return launch_step_t<ST, SCHEME, 2, 8>(v, src, dst, a, s);
     default: return launch_step_t<ST, SCHEME, 2, 10>(v, src, dst, a, s);
     }
@@ -1956,7 +2021,9 @@ cudaError_t launch_step_batch(int config, const BatchEntry* ent, const int64_t* 
     switch (config) {
     case 0: return launch_step_batch_t<ST, 4, 3>(ent, brick_start, n_dom, total_bricks, args, coll, parity, s);
     case 1: return launch_step_batch_t<ST, 2, 7>(ent, brick_start, n_dom, total_bricks, args, coll, parity, s);
-    case 2: return launch_step_batch_t<ST, 2, 6>(ent, brick_start, n_dom, total_bricks, args, coll, parity, s);
+    case 2:  // the default, by size as for a single domain
+        return total_bricks > LARGE_BRICKS ? launch_step_batch_t<ST, 2, 8>(ent, brick_start, n_dom, total_bricks, args, coll, parity, s)
+                                           : launch_step_batch_t<ST, 2, 6>(ent, brick_start, n_dom, total_bricks, args, coll, parity, s);
     case 3: return launch_step_batch_t<ST, 2, 8>(ent, brick_start, n_dom, total_bricks, args, coll, parity, s);
     default: return launch_step_batch_t<ST, 2, 10>(ent, brick_start, n_dom, total_bricks, args, coll, parity, s);
     }

@@ -21,9 +21,9 @@ from paper_2101_11107_gb300 import lbm  # noqa: E402
 oracle.set_threads(min(16, os.cpu_count() or 1))
 
 
-def porous(fluid_fraction, seed):
+def porous(fluid_fraction, seed, shape=(16, 20, 24)):
     rng = np.random.default_rng(seed)
-    mask = (rng.random((16, 20, 24)) < fluid_fraction).astype(np.uint8)
+    mask = (rng.random(shape) < fluid_fraction).astype(np.uint8)
     mask[:, 8:12, :] = 1  # an open channel: bricks without a wall
     mask[4:8] = 1
     links = I.wall_links(mask, lambda p: np.ones(p.shape[:-1]), periodic=(1, 1, 1), iters=1)
@@ -66,6 +66,25 @@ def test_every_configuration_gives_the_same_bits(storage, collision):
             d.set_launch_config(config)
             d.step(30)
             out.append(d.macroscopic())
+            d.close()
+    assert np.abs(out[0][1]).max() > 0
+    for rho, u in out[1:]:
+        assert np.array_equal(rho, out[0][0]) and np.array_equal(u, out[0][1])
+
+
+@pytest.mark.parametrize("storage", ["fp32", "fp16"])
+def test_large_domain_gives_the_same_bits(storage):
+    """A domain of more than 8192 bricks runs kernels of its own (fewer links held in registers, another default
+    register budget); the two-cell kernels and A-B are the comparison."""
+    g = porous(0.6, 13, shape=(64, 84, 128))
+    out = []
+    for scheme, configs in (("esoteric", (6, 0, 1, 2, 3, 4)), ("ab", (0, 2, 4))):
+        for config in configs:
+            d = lbm.Domain.from_geometry(g, scheme=scheme, storage=storage)
+            assert d.info()["n_bricks"] > 8192
+            d.set_launch_config(config)
+            d.step(7)
+            out.append(d.macroscopic(dense=False))
             d.close()
     assert np.abs(out[0][1]).max() > 0
     for rho, u in out[1:]:
