@@ -230,26 +230,42 @@ __device__ __forceinline__ void scale_out2(float2 (&d)[Q])
         if (out_factor<ST, X>(i) != 1.0f) d[i] = __fmul2_rn(d[i], make_float2(out_factor<ST, X>(i), out_factor<ST, X>(i)));
 }
 
+// Programmatic dependent launch between consecutive steps: a step kernel lets the next one start as
+// soon as all its own CTAs are running (pdl_trigger), and the next one loads what no step writes (cell
+// words, records, brick rows) before it waits for this one's populations to be complete and visible
+// (pdl_wait).  Every thread waits before it reads or writes a population, and a kernel ends only after
+// its waiting threads, so the order of more than two kernels follows.  Populations are read with plain
+// loads (not the read-only path: another step may still be writing when a kernel starts).  Both are
+// no-ops in a launch without the attribute.  The step is bound by latency on small domains: the launch
+// gap and the index loads of one step hide behind the tail of the one before.  Measured, per step:
+// 32x32x64 pipe 5.9 -> 4.05 us, 150 k cell aneurysm 14.0 -> 11.9 us, 633 k cell pipe 26.3 -> 24.2 us
+// (FP32 twist), 31.6 -> 29.6 us (A-B), 21.8 -> 19.9 us (FP16); batch of 178 k cells 20.5 -> 19.3 us.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ------------------------------------------------------------------------------ streaming
 // A-B pull: f_i(x, n) = f*_i(x - c_i, n - 1) from `src`; a wall link reads the cell's own
 // opposite slot (halfway bounce-back f_i(x, n) = f*_opp(i)(x, n - 1)).
 template <int ST>
-__device__ __forceinline__ void fetch_ab(const void* __restrict__ src, uint32_t n, const int32_t* nbrow,
-                                         uint32_t slot, uint32_t wm, float (&d)[Q])
+__device__ __forceinline__ void fetch_ab(const void* src, uint32_t n, const int32_t* nbrow, uint32_t slot, uint32_t wm,
+                                         float (&d)[Q])
 {
     const int l = (int)(slot & (BRICK_CELLS - 1));
     const int lx = l & (BX - 1), ly = (l >> LBX) & (BY - 1), lz = l >> (LBX + LBY);
+    uint32_t off[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
         const int sx = lx - cx_of(i), sy = ly - cy_of(i), sz = lz - cz_of(i);
         // sx in [-1, BX]: the arithmetic shift gives the brick offset -1, 0 or +1
         const int ob = 13 + (sx >> LBX) + 3 * (sy >> LBY) + 9 * (sz >> LBZ);
-        const uint32_t nb = (uint32_t)nbrow[ob];
+        const uint32_t nb = (uint32_t)__ldg(nbrow + ob);
         const uint32_t s = nb * BRICK_CELLS + (uint32_t)brick_local(sx & (BX - 1), sy & (BY - 1), sz & (BZ - 1));
         const bool wall = (wm >> i) & 1u;
-        const uint32_t off = wall ? (uint32_t)(Q - 1 - i) * n + slot : (uint32_t)i * n + s;
-        d[i] = LBM_IN_RANGE(off, (uint64_t)Q * n, 1) ? Store<ST>::load_h(src, off) : 0.0f;
+        off[i] = wall ? (uint32_t)(Q - 1 - i) * n + slot : (uint32_t)i * n + s;
     }
+    pdl_wait();
+#pragma unroll
+    for (int i = 0; i < Q; ++i) d[i] = LBM_IN_RANGE(off[i], (uint64_t)Q * n, 1) ? Store<ST>::load_rw_h(src, off[i]) : 0.0f;
     scale_in<ST>(d);
 }
 
@@ -473,12 +489,10 @@ __device__ __forceinline__ uint32_t wall_rules(const DomainView& v, const void* 
     if (kind == KIND_BOUZIDI) {
         const uint32_t off = (uint32_t)(aux >= 0 ? aux : v.aux[slot]);
         // A direction's rule reads d_i and, only when opp(i) has no link, d_opp(i), which no other
-        // direction's rule changes: the order of the directions does not matter.  The twist takes
-        // the links of nine directions at a time (their q and f*_a requested before the first is
-        // used: one memory latency per group, not per link; -26% per step on a 128^3 aneurysm);
-        // A-B, whose f*_a come from the other array, keeps one direction at a time (the grouped
-        // form spills in its 64- to 80-register configurations and was 2% slower on the pipe).
-        constexpr int GS = SCHEME == LBM_SCHEME_ESOTERIC ? 9 : 1;
+        // direction's rule changes: the order of the directions does not matter.  The links of nine
+        // directions at a time (their coefficients and f*_a requested before the first is used: one memory
+        // latency per group, not per link; the A-B exports of a 48 k cell vessel took 13 us link by link).
+        constexpr int GS = 9;
 #pragma unroll
         for (int g = 0; g < Q / GS; ++g) {
             float qg[GS], fg[GS];
@@ -967,37 +981,27 @@ __device__ __forceinline__ void set_own_rate(LevelArgs& la, float s2)
 }
 
 // ------------------------------------------------------------------------------ gather (read-only)
-// Populations of level n of one fluid cell, for the export and diagnostics kernels.
+// Populations of level n of one fluid cell, for the export and diagnostics kernels.  These are programmatic
+// dependents of the step before them: their index tables load while it drains (pdl_wait is in here).
 template <int ST, int SCHEME>
 __device__ __forceinline__ void gather(const DomainView& v, const void* src, uint32_t slot, uint32_t word,
                                        const LevelArgs& a, float (&d)[Q])
 {
     const uint32_t wm = word & WORD_WALL_MASK;
     const uint32_t n = (uint32_t)v.n_slots;
+    const int32_t aux = __ldg(v.aux + slot);
     if (SCHEME == LBM_SCHEME_ESOTERIC) {
         uint32_t cs[8];
         corner_slots(v.nb8 + (slot / BRICK_CELLS) * 8, slot, cs);
-        fetch_et<ST, false>(src, n, cs, wm, a.parity, d);
+        pdl_wait();
+        fetch_et<ST, true>(src, n, cs, wm, a.parity, d);
     } else {
         fetch_ab<ST>(src, n, v.nbr + (slot / BRICK_CELLS) * Q, slot, wm, d);
     }
-    if (wm) wall_rules<ST, SCHEME>(v, src, slot, word, a, d);
+    if (wm) wall_rules<ST, SCHEME>(v, src, slot, word, a, d, aux);
 }
 
 // ------------------------------------------------------------------------------ kernels
-// Programmatic dependent launch between consecutive steps: a step kernel lets the next one start as
-// soon as all its own CTAs are running (pdl_trigger), and the next one loads what no step writes (cell
-// words, records, brick rows) before it waits for this one's populations to be complete and visible
-// (pdl_wait).  Every thread waits before it reads or writes a population, and a kernel ends only after
-// its waiting threads, so the order of more than two kernels follows.  Populations are read with plain
-// loads (not the read-only path: another step may still be writing when a kernel starts).  Both are
-// no-ops in a launch without the attribute.  The step is bound by latency on small domains: the launch
-// gap and the index loads of one step hide behind the tail of the one before.  Measured, per step:
-// 32x32x64 pipe 5.9 -> 4.05 us, 150 k cell aneurysm 14.0 -> 11.9 us, 633 k cell pipe 26.3 -> 24.2 us
-// (FP32 twist), 31.6 -> 29.6 us (A-B), 21.8 -> 19.9 us (FP16); batch of 178 k cells 20.5 -> 19.3 us.
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 // Rounds of links a warp holds in registers: six cover every run of the vessels, so no warp of a small
 // domain, whose step is as long as its slowest warp, waits for the reloading loop (25 k cells: 6.5 -> 5.3 us,
 // 150 k: 10.3 -> 9.5 us against three); on a large domain the warps hide one another's latency and the fewer
@@ -1688,29 +1692,47 @@ __global__ void __launch_bounds__(256)
 }
 
 // FP64 diagnostics: per-block partial sums in a fixed order; one block then reduces the
-// partials in a fixed order (reproducible run to run).
+// partials in a fixed order (reproducible run to run).  The FP64 pipe is narrow (a warp-wide double addition
+// takes about 16 cycles of an SM), so it gets the mass sum and the few flux terms only: the largest speed is
+// kept as its square and compared as integers (the bits of non-negative doubles order like their values; one
+// square root at the end, which is monotonic, gives the same number), the non-finite cells are
+// counted as integers, and a warp without open cells leaves the flux sums out.
 constexpr int DIAG_THREADS = 256;
-constexpr int DIAG_FIELDS = 5;  // mass, flux_in, flux_out, max|u|, non-finite count
+constexpr int DIAG_FIELDS = 5;  // mass, flux_in, flux_out, max |u|^2, non-finite count
 
-__device__ __forceinline__ void block_reduce5(double (&x)[DIAG_FIELDS], double* sh)
+struct Diag {
+    double mass, in, out;
+    unsigned long long u2;  // bits of max |u|^2
+    unsigned int bad;
+};
+__device__ __forceinline__ void diag_add(Diag& x, const Diag& y)
+{
+    x.mass += y.mass;
+    x.in += y.in;
+    x.out += y.out;
+    x.u2 = x.u2 > y.u2 ? x.u2 : y.u2;
+    x.bad += y.bad;
+}
+// the block's total in thread 0, in a fixed order (every warp's tree, then the warps in turn)
+__device__ __forceinline__ void block_reduce(Diag& x, Diag* sh)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool flux = __any_sync(0xffffffffu, x.in != 0.0 || x.out != 0.0);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
-#pragma unroll
-        for (int f = 0; f < DIAG_FIELDS; ++f) {
-            const double o = __shfl_down_sync(0xffffffffu, x[f], off);
-            x[f] = (f == 3) ? fmax(x[f], o) : x[f] + o;
+        x.mass += __shfl_down_sync(0xffffffffu, x.mass, off);
+        const unsigned long long o = __shfl_down_sync(0xffffffffu, x.u2, off);
+        x.u2 = x.u2 > o ? x.u2 : o;
+        if (flux) {
+            x.in += __shfl_down_sync(0xffffffffu, x.in, off);
+            x.out += __shfl_down_sync(0xffffffffu, x.out, off);
         }
     }
-    if (lane == 0)
-        for (int f = 0; f < DIAG_FIELDS; ++f) sh[warp * DIAG_FIELDS + f] = x[f];
+    x.bad = __reduce_add_sync(0xffffffffu, x.bad);
+    if (lane == 0) sh[warp] = x;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < DIAG_THREADS / 32; ++w)
-            for (int f = 0; f < DIAG_FIELDS; ++f)
-                x[f] = (f == 3) ? fmax(x[f], sh[w * DIAG_FIELDS + f]) : x[f] + sh[w * DIAG_FIELDS + f];
-    }
+    if (threadIdx.x == 0)
+        for (int w = 1; w < DIAG_THREADS / 32; ++w) diag_add(x, sh[w]);
 }
 
 template <int ST, int SCHEME>
@@ -1718,8 +1740,9 @@ __global__ void __launch_bounds__(DIAG_THREADS)
     k_diagnostics(DomainView v, const void* src, LevelArgs a, const int32_t* fl_slot, int64_t n_fluid,
                   double* partials)
 {
-    __shared__ double sh[(DIAG_THREADS / 32) * DIAG_FIELDS];
-    double x[DIAG_FIELDS] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    __shared__ Diag sh[DIAG_THREADS / 32];
+    Diag x{0.0, 0.0, 0.0, 0ull, 0u};
+    pdl_trigger();
     const int64_t k = (int64_t)blockIdx.x * DIAG_THREADS + threadIdx.x;
     if (k < n_fluid) {
         const uint32_t slot = (uint32_t)fl_slot[k];
@@ -1729,23 +1752,30 @@ __global__ void __launch_bounds__(DIAG_THREADS)
         const Moments M = moments(d, a.g);
         const bool finite = isfinite(M.rho) && isfinite(M.ux) && isfinite(M.uy) && isfinite(M.uz);
         if (finite) {
-            x[0] = (double)M.rho;
+            x.mass = (double)M.rho;
             const int kind = (int)((word >> WORD_KIND_SHIFT) & 3u);
             if (kind >= KIND_INLET && LBM_IN_RANGE(v.aux[slot], v.n_io, 6)) {
                 const int64_t rec = v.aux[slot];
                 const int ax = v.io_axis[rec];
                 const float un = v.io_sign[rec] * (ax == 0 ? M.ux : ax == 1 ? M.uy : M.uz);
-                if (kind == KIND_INLET) x[1] = (double)M.rho * (double)un;
-                else x[2] = -(double)M.rho * (double)un;
+                if (kind == KIND_INLET) x.in = (double)M.rho * (double)un;
+                else x.out = -(double)M.rho * (double)un;
             }
-            x[3] = sqrt((double)M.ux * M.ux + (double)M.uy * M.uy + (double)M.uz * M.uz);
+            x.u2 = (unsigned long long)__double_as_longlong((double)M.ux * M.ux + (double)M.uy * M.uy + (double)M.uz * M.uz);
         } else {
-            x[4] = 1.0;
+            x.bad = 1u;
         }
     }
-    block_reduce5(x, sh);
-    if (threadIdx.x == 0)
-        for (int f = 0; f < DIAG_FIELDS; ++f) partials[(int64_t)blockIdx.x * DIAG_FIELDS + f] = x[f];
+    block_reduce(x, sh);
+    if (threadIdx.x == 0) {
+        if (n_fluid == 0) pdl_wait();  // no cell has waited: the partials are those of the call before
+        double* p = partials + (int64_t)blockIdx.x * DIAG_FIELDS;
+        p[0] = x.mass;
+        p[1] = x.in;
+        p[2] = x.out;
+        p[3] = __longlong_as_double((long long)x.u2);
+        p[4] = (double)x.bad;
+    }
 }
 
 inline int grid_for(int64_t n, int threads) { return (int)((n + threads - 1) / threads); }
@@ -1869,7 +1899,7 @@ cudaError_t launch_step(int scheme, int config, const DomainView& v, const void*
                                          : launch_step_scheme<ST, LBM_SCHEME_AB>(config, v, src, dst, a, s);
 }
 
-// the export and the correction run one thread per fluid cell; with small CTAs a domain of a few
+// the export, the means and the correction run one thread per fluid cell; with small CTAs a domain of a few
 // ten thousand cells still spreads over every SM (its latency chains overlap on all of them)
 constexpr int PER_CELL_THREADS = 64;
 
@@ -1880,12 +1910,10 @@ cudaError_t launch_macroscopic(int scheme, const DomainView& v, const void* src,
 {
     if (n_fluid == 0) return cudaSuccess;
     if (scheme == LBM_SCHEME_ESOTERIC)
-        k_macroscopic<ST, LBM_SCHEME_ESOTERIC><<<grid_for(n_fluid, PER_CELL_THREADS), PER_CELL_THREADS, 0, s>>>(v, src, a, fl_slot, fl_box,
-                                                                                  n_fluid, dense, rho, u, n_out);
-    else
-        k_macroscopic<ST, LBM_SCHEME_AB><<<grid_for(n_fluid, PER_CELL_THREADS), PER_CELL_THREADS, 0, s>>>(v, src, a, fl_slot, fl_box, n_fluid,
-                                                                            dense, rho, u, n_out);
-    return cudaGetLastError();
+        return launch_pdl(k_macroscopic<ST, LBM_SCHEME_ESOTERIC>, grid_for(n_fluid, PER_CELL_THREADS), PER_CELL_THREADS, 0, s, v,
+                          src, a, fl_slot, fl_box, n_fluid, dense, rho, u, n_out);
+    return launch_pdl(k_macroscopic<ST, LBM_SCHEME_AB>, grid_for(n_fluid, PER_CELL_THREADS), PER_CELL_THREADS, 0, s, v, src, a,
+                      fl_slot, fl_box, n_fluid, dense, rho, u, n_out);
 }
 
 template <int ST>
@@ -1894,10 +1922,10 @@ cudaError_t launch_mean_sample(int scheme, const DomainView& v, const void* src,
 {
     if (n_fluid == 0) return cudaSuccess;
     if (scheme == LBM_SCHEME_ESOTERIC)
-        k_mean_sample<ST, LBM_SCHEME_ESOTERIC><<<grid_for(n_fluid, 256), 256, 0, s>>>(v, src, a, fl_slot, n_fluid, sums);
-    else
-        k_mean_sample<ST, LBM_SCHEME_AB><<<grid_for(n_fluid, 256), 256, 0, s>>>(v, src, a, fl_slot, n_fluid, sums);
-    return cudaGetLastError();
+        return launch_pdl(k_mean_sample<ST, LBM_SCHEME_ESOTERIC>, grid_for(n_fluid, PER_CELL_THREADS), PER_CELL_THREADS, 0, s, v,
+                          src, a, fl_slot, n_fluid, sums);
+    return launch_pdl(k_mean_sample<ST, LBM_SCHEME_AB>, grid_for(n_fluid, PER_CELL_THREADS), PER_CELL_THREADS, 0, s, v, src, a,
+                      fl_slot, n_fluid, sums);
 }
 
 template <int ST>
@@ -1933,10 +1961,8 @@ cudaError_t launch_diagnostics(int scheme, const DomainView& v, const void* src,
 {
     const int nb = (int)diagnostics_blocks(n_fluid);
     if (scheme == LBM_SCHEME_ESOTERIC)
-        k_diagnostics<ST, LBM_SCHEME_ESOTERIC><<<nb, DIAG_THREADS, 0, s>>>(v, src, a, fl_slot, n_fluid, partials);
-    else
-        k_diagnostics<ST, LBM_SCHEME_AB><<<nb, DIAG_THREADS, 0, s>>>(v, src, a, fl_slot, n_fluid, partials);
-    return cudaGetLastError();
+        return launch_pdl(k_diagnostics<ST, LBM_SCHEME_ESOTERIC>, nb, DIAG_THREADS, 0, s, v, src, a, fl_slot, n_fluid, partials);
+    return launch_pdl(k_diagnostics<ST, LBM_SCHEME_AB>, nb, DIAG_THREADS, 0, s, v, src, a, fl_slot, n_fluid, partials);
 }
 
 template <int ST>

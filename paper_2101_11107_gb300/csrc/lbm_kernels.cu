@@ -29,20 +29,20 @@ namespace {
 __global__ void __launch_bounds__(dev::DIAG_THREADS)
     k_diagnostics_final(const double* partials, int64_t n_blocks, lbm_diagnostics* out)
 {
-    __shared__ double sh[(dev::DIAG_THREADS / 32) * dev::DIAG_FIELDS];
-    double x[dev::DIAG_FIELDS] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int64_t b = threadIdx.x; b < n_blocks; b += dev::DIAG_THREADS)
-        for (int f = 0; f < dev::DIAG_FIELDS; ++f) {
-            const double p = partials[b * dev::DIAG_FIELDS + f];
-            x[f] = (f == 3) ? fmax(x[f], p) : x[f] + p;
-        }
-    dev::block_reduce5(x, sh);
+    __shared__ dev::Diag sh[dev::DIAG_THREADS / 32];
+    dev::Diag x{0.0, 0.0, 0.0, 0ull, 0u};
+    dev::pdl_wait();
+    for (int64_t b = threadIdx.x; b < n_blocks; b += dev::DIAG_THREADS) {
+        const double* p = partials + b * dev::DIAG_FIELDS;
+        dev::diag_add(x, dev::Diag{p[0], p[1], p[2], (unsigned long long)__double_as_longlong(p[3]), (unsigned int)p[4]});
+    }
+    dev::block_reduce(x, sh);
     if (threadIdx.x == 0) {
-        out->mass = x[0];
-        out->flux_in = x[1];
-        out->flux_out = x[2];
-        out->max_u = x[3];
-        out->n_nonfinite = (int64_t)x[4];
+        out->mass = x.mass;
+        out->flux_in = x.in;
+        out->flux_out = x.out;
+        out->max_u = sqrt(__longlong_as_double((long long)x.u2));
+        out->n_nonfinite = (int64_t)x.bad;
     }
 }
 }  // namespace
@@ -93,8 +93,7 @@ cudaError_t launch_halo_copy(int bytes_per_value, bool pack, void* pop, int64_t 
 cudaError_t launch_diagnostics_final(const double* partials, int64_t n_blocks, lbm_diagnostics* out,
                                      cudaStream_t stream)
 {
-    k_diagnostics_final<<<1, dev::DIAG_THREADS, 0, stream>>>(partials, n_blocks, out);
-    return cudaGetLastError();
+    return dev::launch_pdl(k_diagnostics_final, 1, dev::DIAG_THREADS, 0, stream, partials, n_blocks, out);
 }
 
 }  // namespace lbm
