@@ -118,6 +118,7 @@ struct LevelArgs {
     float rho_out;
     float drho_out;  // rho_out - 1, rounded once from FP64
     int parity;      // n & 1 (esoteric twist)
+    int backwards;   // the step sweeps the bricks from the last to the first (set by its launcher)
     int coll;        // collision kernel: COLL_CHM, COLL_CHM_FAST (every 3rd..6th-order rate is
                      // 1: the step kernel skips those moments), COLL_SRT2, COLL_TRT2
     float wm;        // SRT2 / TRT2: rate of the odd parts (SRT2: = s2)

@@ -75,7 +75,8 @@ def test_every_configuration_gives_the_same_bits(storage, collision):
 @pytest.mark.parametrize("storage", ["fp32", "fp16"])
 def test_large_domain_gives_the_same_bits(storage):
     """A domain of more than 8192 bricks runs kernels of its own (fewer links held in registers, another default
-    register budget); the two-cell kernels and A-B are the comparison."""
+    register budget), and a state of more than 64 MB is swept backwards on odd levels; the two-cell kernels,
+    A-B and, in FP16, the twist (40 MB, one order) are the comparison."""
     g = porous(0.6, 13, shape=(64, 84, 128))
     out = []
     for scheme, configs in (("esoteric", (6, 0, 1, 2, 3, 4)), ("ab", (0, 2, 4))):

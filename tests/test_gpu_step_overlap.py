@@ -49,3 +49,21 @@ def test_captured_steps_replay(scheme):
     (ra, ua), (rb, ub) = a.macroscopic(), b.macroscopic()
     assert np.abs(ua).max() > 0
     assert np.array_equal(ra, rb) and np.array_equal(ua, ub)
+
+
+@pytest.mark.parametrize("graph_steps", [1, 2, 5])
+def test_batch_chunks_in_flight(graph_steps):
+    """Many short batch chunks enqueued without waiting, each with its own level arguments (pulsatile inflow and
+    force): the fields of the domains stepped alone."""
+    gs = [I.aneurysm(20 + k, edge=e, period=37.0 + 5 * k, reynolds=40.0, wave_seed=50 + k) for k, e in enumerate((48, 64))]
+    doms, alone = ([lbm.Domain.from_geometry(g, storage="fp32") for g in gs] for _ in range(2))
+    batch = lbm.Batch(doms, graph_steps=graph_steps)
+    for n in (graph_steps, 23, 1, 16):
+        batch.step(n)
+    batch.sync()
+    for d, a in zip(doms, alone):
+        a.step(graph_steps + 40)
+        assert d.time == a.time
+        (r1, u1), (r2, u2) = d.macroscopic(), a.macroscopic()
+        assert np.abs(u1).max() > 0 and np.array_equal(r1, r2) and np.array_equal(u1, u2)
+    batch.close()
