@@ -54,31 +54,27 @@ NOMINAL_HBM_GBS = 8000.0  # the metric's roofline denominator (bytes per fluid-c
 # configuration); reported only for the configuration the bench runs, None for any other.  An
 # entry is removed whenever the kernel it was taken on changes.
 K_STEP_TRAFFIC = {
-    ("womersley", "fp32", "ab", "128x10"): (125_738_240, "k_step<fp32, A-B, 2 bricks, 10 CTAs/SM, default rates> (88.68 MB read, 37.06 MB written)"),
-    ("womersley", "fp32", "ab", "128x6"): (121_100_544, "k_step<fp32, A-B, 2 bricks, 6 CTAs/SM, default rates> (86.99 MB read, 34.11 MB written)"),
-    ("womersley", "fp32", "ab", "128x7"): (120_878_592, "k_step<fp32, A-B, 2 bricks, 7 CTAs/SM, default rates> (87.03 MB read, 33.85 MB written)"),
-    ("womersley", "fp32", "ab", "128x8"): (120_099_840, "k_step<fp32, A-B, 2 bricks, 8 CTAs/SM, default rates> (86.96 MB read, 33.14 MB written)"),
-    ("womersley", "fp32", "ab", "256x3"): (121_325_824, "k_step<fp32, A-B, 4 bricks, 3 CTAs/SM, default rates> (86.97 MB read, 34.35 MB written)"),
-    ("womersley", "fp32", "esoteric", "128x10"): (116_750_592, "k_step<fp32, twist, 2 bricks, 10 CTAs/SM, default rates, parity 1> (84.08 MB read, 32.68 MB written)"),
-    ("womersley", "fp32", "esoteric", "128x6"): (101_404_160, "k_step<fp32, twist, 2 bricks, 6 CTAs/SM, default rates, parity 1> (82.83 MB read, 18.57 MB written)"),
-    ("womersley", "fp32", "esoteric", "128x7"): (101_440_256, "k_step<fp32, twist, 2 bricks, 7 CTAs/SM, default rates, parity 1> (82.83 MB read, 18.61 MB written)"),
-    ("womersley", "fp32", "esoteric", "128x8"): (106_862_336, "k_step<fp32, twist, 2 bricks, 8 CTAs/SM, default rates, parity 1> (83.17 MB read, 23.69 MB written)"),
-    ("womersley", "fp32", "esoteric", "256x3"): (100_946_944, "k_step<fp32, twist, 4 bricks, 3 CTAs/SM, default rates, parity 1> (82.82 MB read, 18.13 MB written)"),
-    ("womersley", "fp32", "esoteric", "2c128x3"): (101_332_224, "k_step2<fp32, 4 bricks, 3 CTAs/SM> (82.85 MB read, 18.48 MB written)"),
-    ("womersley", "fp32", "esoteric", "2c128x4"): (102_119_680, "k_step2<fp32, 4 bricks, 4 CTAs/SM> (82.90 MB read, 19.22 MB written)"),
-    ("womersley", "fp32", "esoteric", "pipe128x6"): (98_264_576, "k_step_et_pipe<fp32, 2 bricks, 6 CTAs/SM, persistent> (79.99 MB read, 18.27 MB written)"),
-    ("aneurysm512", "fp32", "esoteric", "256x3"): (250_623_744, "k_step<fp32, twist, 4 bricks, 3 CTAs/SM, default rates, parity 1> (165.48 MB read, 85.14 MB written)"),
-    ("aneurysm512", "fp32", "esoteric", "128x6"): (250_743_296, "k_step<fp32, twist, 2 bricks, 6 CTAs/SM, default rates, parity 1> (165.51 MB read, 85.24 MB written)"),
-    ("aneurysm512", "fp32", "esoteric", "128x10"): (285_614_080, "k_step<fp32, twist, 2 bricks, 10 CTAs/SM, default rates, parity 1> (171.06 MB read, 114.56 MB written)"),
-    ("aneurysm512", "fp32", "esoteric", "2c128x4"): (251_746_304, "k_step2<fp32, 4 bricks, 4 CTAs/SM> (165.76 MB read, 85.98 MB written)"),
-    ("aneurysm512", "fp32", "esoteric", "2c128x3"): (250_264_320, "k_step2<fp32, 4 bricks, 3 CTAs/SM> (165.71 MB read, 84.56 MB written)"),
-    ("aneurysm512", "fp32", "esoteric", "pipe128x6"): (245_090_048, "k_step_et_pipe<fp32, 2 bricks, 6 CTAs/SM, persistent> (159.69 MB read, 85.40 MB written)"),
-    ("aneurysm512", "fp32", "esoteric", "128x7"): (250_688_512,
-                                                   "k_step<fp32, twist, 2 bricks, 7 CTAs/SM, default rates, parity 1> "
-                                                   "(165.51 MB read, 85.18 MB written)"),
-    ("aneurysm512", "fp32", "esoteric", "128x8"): (260_912_896,
-                                                   "k_step<fp32, twist, 2 bricks, 8 CTAs/SM, default rates, parity 1> "
-                                                   "(166.24 MB read, 94.67 MB written)"),
+    ("womersley", "fp32", "ab", "256x3"): (120_867_328, "k_step<fp32, A-B, 4 bricks, 3 CTAs/SM, default rates, no links> (89.77 MB read, 31.10 MB written)"),
+    ("womersley", "fp32", "ab", "128x7"): (120_340_992, "k_step<fp32, A-B, 2 bricks, 7 CTAs/SM, default rates, no links> (89.81 MB read, 30.53 MB written)"),
+    ("womersley", "fp32", "ab", "128x6"): (119_857_408, "k_step<fp32, A-B, 2 bricks, 8 CTAs/SM, default rates, no links> (89.75 MB read, 30.10 MB written)"),
+    ("womersley", "fp32", "ab", "128x8"): (120_348_160, "k_step<fp32, A-B, 2 bricks, 8 CTAs/SM, default rates, no links> (89.79 MB read, 30.55 MB written)"),
+    ("womersley", "fp32", "ab", "128x10"): (122_133_760, "k_step<fp32, A-B, 2 bricks, 10 CTAs/SM, default rates, no links> (89.72 MB read, 32.42 MB written)"),
+    ("womersley", "fp32", "esoteric", "256x3"): (97_949_184, "k_step<fp32, twist, 4 bricks, 3 CTAs/SM, default rates, parity 1, no links> (82.82 MB read, 15.13 MB written)"),
+    ("womersley", "fp32", "esoteric", "128x7"): (98_066_432, "k_step<fp32, twist, 2 bricks, 7 CTAs/SM, default rates, parity 1, no links> (82.82 MB read, 15.25 MB written)"),
+    ("womersley", "fp32", "esoteric", "128x6"): (98_080_256, "k_step<fp32, twist, 2 bricks, 8 CTAs/SM, default rates, parity 1, no links> (82.82 MB read, 15.26 MB written)"),
+    ("womersley", "fp32", "esoteric", "128x8"): (98_131_968, "k_step<fp32, twist, 2 bricks, 8 CTAs/SM, default rates, parity 1, no links> (82.81 MB read, 15.32 MB written)"),
+    ("womersley", "fp32", "esoteric", "128x10"): (101_006_080, "k_step<fp32, twist, 2 bricks, 10 CTAs/SM, default rates, parity 1, no links> (82.98 MB read, 18.03 MB written)"),
+    ("womersley", "fp32", "esoteric", "pipe128x6"): (95_522_816, "k_step_et_pipe<fp32, 2 bricks, 6 CTAs/SM, persistent> (79.98 MB read, 15.54 MB written)"),
+    ("womersley", "fp32", "esoteric", "2c128x4"): (98_055_424, "k_step2<fp32, 4 bricks, 4 CTAs/SM> (82.85 MB read, 15.20 MB written)"),
+    ("womersley", "fp32", "esoteric", "2c128x3"): (97_840_128, "k_step2<fp32, 4 bricks, 3 CTAs/SM> (82.86 MB read, 14.98 MB written)"),
+    ("aneurysm512", "fp32", "esoteric", "256x3"): (247_981_312, "k_step<fp32, twist, 4 bricks, 3 CTAs/SM, default rates, parity 1, 3 link rounds> (166.84 MB read, 81.14 MB written)"),
+    ("aneurysm512", "fp32", "esoteric", "128x7"): (253_959_424, "k_step<fp32, twist, 2 bricks, 7 CTAs/SM, default rates, parity 1, 3 link rounds> (167.02 MB read, 86.94 MB written)"),
+    ("aneurysm512", "fp32", "esoteric", "128x6"): (248_477_440, "k_step<fp32, twist, 2 bricks, 8 CTAs/SM, default rates, parity 1, 3 link rounds> (166.83 MB read, 81.64 MB written)"),
+    ("aneurysm512", "fp32", "esoteric", "128x8"): (248_439_040, "k_step<fp32, twist, 2 bricks, 8 CTAs/SM, default rates, parity 1, 3 link rounds> (166.81 MB read, 81.63 MB written)"),
+    ("aneurysm512", "fp32", "esoteric", "128x10"): (271_365_888, "k_step<fp32, twist, 2 bricks, 10 CTAs/SM, default rates, parity 1, 3 link rounds> (167.36 MB read, 104.01 MB written)"),
+    ("aneurysm512", "fp32", "esoteric", "pipe128x6"): (242_021_120, "k_step_et_pipe<fp32, 2 bricks, 6 CTAs/SM, persistent> (159.48 MB read, 82.54 MB written)"),
+    ("aneurysm512", "fp32", "esoteric", "2c128x4"): (246_262_272, "k_step2<fp32, 4 bricks, 4 CTAs/SM> (165.11 MB read, 81.16 MB written)"),
+    ("aneurysm512", "fp32", "esoteric", "2c128x3"): (246_018_816, "k_step2<fp32, 4 bricks, 3 CTAs/SM> (165.18 MB read, 80.84 MB written)"),
 }
 
 

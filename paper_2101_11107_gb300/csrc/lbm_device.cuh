@@ -66,8 +66,8 @@ __device__ __forceinline__ bool dbg_in_range(uint64_t i, uint64_t n, unsigned co
 #endif
 
 // ------------------------------------------------------------------------------ storage
-// FP32 stores d_i; FP16 / BF16 store d_i / w_i.  `load` may use the read-only path (arrays
-// not written by the kernel); `load_rw` is a plain load (the in-place array).
+// FP32 stores d_i; FP16 / BF16 store d_i / w_i.  Loads are plain, not of the read-only path: a kernel may
+// start while the step before it still writes (pdl_wait).
 template <int ST>
 struct Store;
 
@@ -75,11 +75,6 @@ template <>
 struct Store<LBM_STORE_FP32> {
     using T = float;
     static constexpr bool SCALED = false;  // the stored value is d itself
-    static __device__ __forceinline__ float load(const void* p, int, uint32_t off)
-    {
-        return __ldg(static_cast<const float*>(p) + off);
-    }
-    static __device__ __forceinline__ float load_h(const void* p, uint32_t off) { return load(p, 0, off); }
     // with a 256-byte L2 fetch on a miss: a warp reads 128 bytes of a brick's 256-byte plane
     // row and the other half-brick warp (or the neighbour brick's shifted read) the rest, so
     // the second request finds it in L2 (measured: -3% per step cold for the two-cell kernel,
@@ -108,20 +103,12 @@ struct Store<LBM_STORE_FP32> {
 template <>
 struct Store<LBM_STORE_FP16> {
     using T = __half;
-    static __device__ __forceinline__ float load(const void* p, int i, uint32_t off)
-    {
-        return w_of(i) * __half2float(__ldg(static_cast<const __half*>(p) + off));
-    }
     static __device__ __forceinline__ float load_rw(const void* p, int i, uint32_t off)
     {
         return w_of(i) * __half2float(static_cast<const __half*>(p)[off]);
     }
     // the stored h = d / w as a float (the caller multiplies by w_i: scale_in)
     static constexpr bool SCALED = true;
-    static __device__ __forceinline__ float load_h(const void* p, uint32_t off)
-    {
-        return __half2float(__ldg(static_cast<const __half*>(p) + off));
-    }
     static __device__ __forceinline__ float load_rw_h(const void* p, uint32_t off)
     {
         return __half2float(static_cast<const __half*>(p)[off]);
@@ -145,20 +132,12 @@ struct Store<LBM_STORE_FP16> {
 template <>
 struct Store<LBM_STORE_BF16> {
     using T = __nv_bfloat16;
-    static __device__ __forceinline__ float load(const void* p, int i, uint32_t off)
-    {
-        return w_of(i) * __bfloat162float(__ldg(static_cast<const __nv_bfloat16*>(p) + off));
-    }
     static __device__ __forceinline__ float load_rw(const void* p, int i, uint32_t off)
     {
         return w_of(i) * __bfloat162float(static_cast<const __nv_bfloat16*>(p)[off]);
     }
     // the stored h = d / w as a float (the caller multiplies by w_i: scale_in)
     static constexpr bool SCALED = true;
-    static __device__ __forceinline__ float load_h(const void* p, uint32_t off)
-    {
-        return __bfloat162float(__ldg(static_cast<const __nv_bfloat16*>(p) + off));
-    }
     static __device__ __forceinline__ float load_rw_h(const void* p, uint32_t off)
     {
         return __bfloat162float(static_cast<const __nv_bfloat16*>(p)[off]);
@@ -323,7 +302,7 @@ __device__ __forceinline__ void corner_slots(const int32_t* nb8, uint32_t slot, 
 // on a wall link the other slot of the same cell, which holds f*_opp(i)(x, n - 1).
 // PC >= 0 fixes the parity at compile time; with `clean` (warp-uniform: no lane of the warp has a
 // wall link) every plane index is then a constant.
-template <int ST, bool RW, int PC = -1>
+template <int ST, int PC = -1>
 __device__ __forceinline__ void fetch_et(const void* pop, uint32_t n, const uint32_t (&cs)[8], uint32_t wm,
                                          int parity, float (&d)[Q], bool clean = false)
 {
@@ -331,7 +310,7 @@ __device__ __forceinline__ void fetch_et(const void* pop, uint32_t n, const uint
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
             const uint32_t off = (PC ? (uint32_t)(Q - 1 - i) : (uint32_t)i) * n + cs[corner_neg(i)];
-            d[i] = LBM_IN_RANGE(off, (uint64_t)Q * n, 2) ? (RW ? Store<ST>::load_rw_h(pop, off) : Store<ST>::load_h(pop, off))
+            d[i] = LBM_IN_RANGE(off, (uint64_t)Q * n, 2) ? Store<ST>::load_rw_h(pop, off)
                                                         : 0.0f;
         }
         scale_in<ST>(d);
@@ -343,7 +322,7 @@ __device__ __forceinline__ void fetch_et(const void* pop, uint32_t n, const uint
         const uint32_t flip = ((uint32_t)parity ^ (wm >> i)) & 1u;
         const uint32_t dir = flip ? (uint32_t)(Q - 1 - i) : (uint32_t)i;
         const uint32_t off = dir * n + cs[corner_neg(i)];
-        d[i] = LBM_IN_RANGE(off, (uint64_t)Q * n, 2) ? (RW ? Store<ST>::load_rw_h(pop, off) : Store<ST>::load_h(pop, off))
+        d[i] = LBM_IN_RANGE(off, (uint64_t)Q * n, 2) ? Store<ST>::load_rw_h(pop, off)
                                                     : 0.0f;
     }
     scale_in<ST>(d);
@@ -994,7 +973,7 @@ __device__ __forceinline__ void gather(const DomainView& v, const void* src, uin
         uint32_t cs[8];
         corner_slots(v.nb8 + (slot / BRICK_CELLS) * 8, slot, cs);
         pdl_wait();
-        fetch_et<ST, true>(src, n, cs, wm, a.parity, d);
+        fetch_et<ST>(src, n, cs, wm, a.parity, d);
     } else {
         fetch_ab<ST>(src, n, v.nbr + (slot / BRICK_CELLS) * Q, slot, wm, d);
     }
@@ -1183,7 +1162,7 @@ __device__ __forceinline__ void step_cell(const DomainView& v, const void* src, 
         const bool clean = PC >= 0 && __all_sync(0xffffffffu, wm == 0u);
         if (LINKS) links.prefetch(v);
         if (PDL) pdl_wait();
-        if (fluid) fetch_et<ST, true, PC>(dst, n, cs, wm, a.parity, d, clean);
+        if (fluid) fetch_et<ST, PC>(dst, n, cs, wm, a.parity, d, clean);
     } else {
         const int32_t row = __ldg(v.nbr + brick * (uint32_t)Q + (lane < (uint32_t)Q ? lane : 0u));
         if (LINKS) links.prefetch(v);
@@ -1292,8 +1271,8 @@ __global__ void __launch_bounds__(BRICKS * 32, MINB)
     pdl_wait();
     if (!fA && !fB) return;
     float dA[Q], dB[Q];
-    if (fA) fetch_et<ST, true, PC>(pop, n, csA, wA & WORD_WALL_MASK, a.parity, dA, clean);
-    if (fB) fetch_et<ST, true, PC>(pop, n, csB, wB & WORD_WALL_MASK, a.parity, dB, clean);
+    if (fA) fetch_et<ST, PC>(pop, n, csA, wA & WORD_WALL_MASK, a.parity, dA, clean);
+    if (fB) fetch_et<ST, PC>(pop, n, csB, wB & WORD_WALL_MASK, a.parity, dB, clean);
     const uint32_t halfA =
         (fA && (wA & WORD_WALL_MASK)) ? wall_rules<ST, LBM_SCHEME_ESOTERIC>(v, nullptr, slotA, wA, a, dA, xA) : 0u;
     const uint32_t halfB =
