@@ -223,6 +223,14 @@ __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.lau
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // ------------------------------------------------------------------------------ streaming
+template <int ST>
+__device__ __forceinline__ void fetch_ab_at(const void* src, uint32_t n, const uint32_t (&off)[Q], float (&d)[Q])
+{
+#pragma unroll
+    for (int i = 0; i < Q; ++i) d[i] = LBM_IN_RANGE(off[i], (uint64_t)Q * n, 1) ? Store<ST>::load_rw_h(src, off[i]) : 0.0f;
+    scale_in<ST>(d);
+}
+
 // A-B pull: f_i(x, n) = f*_i(x - c_i, n - 1) from `src`; a wall link reads the cell's own
 // opposite slot (halfway bounce-back f_i(x, n) = f*_opp(i)(x, n - 1)).
 template <int ST>
@@ -243,33 +251,31 @@ __device__ __forceinline__ void fetch_ab(const void* src, uint32_t n, const int3
         off[i] = wall ? (uint32_t)(Q - 1 - i) * n + slot : (uint32_t)i * n + s;
     }
     pdl_wait();
-#pragma unroll
-    for (int i = 0; i < Q; ++i) d[i] = LBM_IN_RANGE(off[i], (uint64_t)Q * n, 1) ? Store<ST>::load_rw_h(src, off[i]) : 0.0f;
-    scale_in<ST>(d);
+    fetch_ab_at<ST>(src, n, off, d);
 }
 
 // A-B pull in the step kernel: the brick's 27-entry neighbour row is held by lanes 0..26 of the
 // warp (a warp covers half of one brick) and handed out with shuffles, so no CTA barrier or
-// shared staging is needed.  All 32 lanes run the shuffles; only fluid lanes load (plain loads: a
-// step may start while the one before it still writes, so its source is not read-only for it).
-template <int ST>
-__device__ __forceinline__ void fetch_ab_shfl(const void* src, uint32_t n, int32_t row_lane,
-                                              uint32_t slot, uint32_t wm, bool fluid, float (&d)[Q])
+// shared staging is needed.  All 32 lanes must call this; the offset of direction i.
+__device__ __forceinline__ uint32_t ab_offset_shfl(uint32_t n, int32_t row_lane, uint32_t slot, uint32_t wm, int i)
 {
     const int l = (int)(slot & (BRICK_CELLS - 1));
     const int lx = l & (BX - 1), ly = (l >> LBX) & (BY - 1), lz = l >> (LBX + LBY);
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        const int sx = lx - cx_of(i), sy = ly - cy_of(i), sz = lz - cz_of(i);
-        const int ob = 13 + (sx >> LBX) + 3 * (sy >> LBY) + 9 * (sz >> LBZ);
-        const uint32_t nb = (uint32_t)__shfl_sync(0xffffffffu, row_lane, ob);
-        const uint32_t s = nb * BRICK_CELLS + (uint32_t)brick_local(sx & (BX - 1), sy & (BY - 1), sz & (BZ - 1));
-        const bool wall = (wm >> i) & 1u;
-        const uint32_t off = wall ? (uint32_t)(Q - 1 - i) * n + slot : (uint32_t)i * n + s;
-        if (fluid) d[i] = LBM_IN_RANGE(off, (uint64_t)Q * n, 1) ? Store<ST>::load_rw_h(src, off) : 0.0f;
-    }
-    if (fluid) scale_in<ST>(d);
+    const int sx = lx - cx_of(i), sy = ly - cy_of(i), sz = lz - cz_of(i);
+    const int ob = 13 + (sx >> LBX) + 3 * (sy >> LBY) + 9 * (sz >> LBZ);
+    const uint32_t nb = (uint32_t)__shfl_sync(0xffffffffu, row_lane, ob);
+    const uint32_t s = nb * BRICK_CELLS + (uint32_t)brick_local(sx & (BX - 1), sy & (BY - 1), sz & (BZ - 1));
+    return ((wm >> i) & 1u) ? (uint32_t)(Q - 1 - i) * n + slot : (uint32_t)i * n + s;
 }
+
+// Whether an A-B step forms all its offsets before its first load.  Loads are plain (a step may start while the
+// one before it still writes) and stay in order with the shuffles, and a shuffle between two loads waits
+// for the loads before it: few are in flight at a time.  Per step, one by one -> all first: 2.7 M cell Bouzidi
+// pipe FP16 170 -> 98 us, FP16 TRT 197 -> 108 us, FP32 TRT 124 -> 118 us; 633 k cell pipe FP16 TRT 43.4 -> 25.3 us,
+// FP32 TRT 31.9 -> 29.0 us.  FP32 with the default rates keeps them one by one: 109 us, and 116 us all first
+// (2.7 M cells); 26.8 and 26.9 us (633 k cells).
+template <int ST, int COLL>
+__host__ __device__ constexpr bool ab_offsets_first() { return !(ST == LBM_STORE_FP32 && COLL == COLL_CHM_FAST); }
 
 // Twist corner slots in the step kernel: lanes hold the brick's nb8 row (lane & 7).
 __device__ __forceinline__ void corner_slots_shfl(int32_t row_lane, uint32_t slot, uint32_t (&cs)[8])
@@ -1165,9 +1171,23 @@ __device__ __forceinline__ void step_cell(const DomainView& v, const void* src, 
         if (fluid) fetch_et<ST, PC>(dst, n, cs, wm, a.parity, d, clean);
     } else {
         const int32_t row = __ldg(v.nbr + brick * (uint32_t)Q + (lane < (uint32_t)Q ? lane : 0u));
+        constexpr bool FIRST = ab_offsets_first<ST, COLL>();
+        uint32_t off[Q];
+        if (FIRST)
+#pragma unroll
+            for (int i = 0; i < Q; ++i) off[i] = ab_offset_shfl(n, row, slot, wm, i);
         if (LINKS) links.prefetch(v);
         if (PDL) pdl_wait();
-        fetch_ab_shfl<ST>(src, n, row, slot, wm, fluid, d);
+        if (FIRST) {
+            if (fluid) fetch_ab_at<ST>(src, n, off, d);
+        } else {
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                off[i] = ab_offset_shfl(n, row, slot, wm, i);
+                if (fluid) d[i] = LBM_IN_RANGE(off[i], (uint64_t)Q * n, 1) ? Store<ST>::load_rw_h(src, off[i]) : 0.0f;
+            }
+            if (fluid) scale_in<ST>(d);
+        }
     }
     if (LINKS && links.any()) {
         links.issue(v, src, slot0);

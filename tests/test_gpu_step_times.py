@@ -1,0 +1,46 @@
+"""Times that must stand in a known relation to one another, whatever the GPU's clock: a step that moves half
+the bytes of another is not the slower one."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from paper_2101_11107_gb300 import inputs as I  # noqa: E402
+from paper_2101_11107_gb300 import lbm  # noqa: E402
+
+
+def gpu_us(fn, n=1, repeats=7):
+    """Median device time of one of the n things that fn does."""
+    fn()
+    out = []
+    for _ in range(repeats):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        torch.cuda.synchronize()
+        a.record()
+        fn()
+        b.record()
+        torch.cuda.synchronize()
+        out.append(a.elapsed_time(b) * 1e3 / n)
+    return float(np.median(out))
+
+
+@pytest.fixture(scope="module")
+def large_pipe():
+    """19 k bricks, 1.2 M cells, interpolated walls: larger than L2 in every storage with two arrays."""
+    return I.pipe(96, 96, 192, 44.3, tau=0.55, gamp=(0.0, 0.0, 1e-5), gomega=0.001, bouzidi=True)
+
+
+@pytest.mark.parametrize("storage", ["fp16", "bf16"])
+@pytest.mark.parametrize("collision", ["chm", "trt2"])
+def test_16_bit_ab_step_is_no_slower_than_fp32(large_pipe, collision, storage):
+    """Half the bytes and the same number of loads (5% for the spread of the times)."""
+    t = {}
+    for st in ("fp32", storage):
+        d = lbm.Domain.from_geometry(large_pipe, storage=st, scheme="ab", collision=collision)
+        t[st] = gpu_us(lambda: d.step(40), 40)
+        d.close()
+    assert t[storage] <= 1.05 * t["fp32"], t
