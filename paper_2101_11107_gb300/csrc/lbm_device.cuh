@@ -1431,6 +1431,10 @@ __global__ void __launch_bounds__(BRICKS * BRICK_CELLS, MINB)
 // reads what neighbouring CTAs wrote.  Every wait at the barrier is bounded by `limit_ns` of the
 // global timer: a CTA that gives up raises bar->fail and every CTA leaves at its next barrier, so
 // a chunk that cannot complete ends instead of hanging (the host then reports LBM_ERR_TIMEOUT).
+// One body for both parities and a budget of 80 registers (6 CTAs per SM): two bodies, one per parity, with six
+// link rounds in 64 registers spilled 2 KB a thread.  Per step, default rates, two bodies in 64 registers -> this:
+// 2 vessels FP16 12.6 -> 8.1 us, 8 vessels 34.3 -> 20.8 us, 16 vessels 56.6 -> 34.2 us (FP32 60.4 -> 34.2 us); one
+// body in 64 registers with three rounds: 10.8, 23.7 and 35.7 us.
 __device__ __forceinline__ uint64_t global_ns()
 {
     uint64_t t;
@@ -1471,7 +1475,7 @@ __device__ __forceinline__ bool grid_barrier(GridBarrier* bar, unsigned int targ
     return ok != 0;
 }
 
-template <int ST, int BRICKS, int MINB, int COLL, int P0>
+template <int ST, int BRICKS, int MINB, int COLL>
 __global__ void __launch_bounds__(BRICKS * BRICK_CELLS, MINB)
     k_step_batch_persistent(const BatchEntry* __restrict__ ent, const int64_t* __restrict__ brick_start, int n_dom,
                             const LevelArgs* __restrict__ args, int steps, GridBarrier* bar, unsigned int* tickets,
@@ -1502,15 +1506,8 @@ __global__ void __launch_bounds__(BRICKS * BRICK_CELLS, MINB)
                 const LevelArgs a = args[(size_t)s * n_dom + lo];
                 const uint32_t slot =
                     (uint32_t)((gbrick - __ldg(brick_start + lo)) * BRICK_CELLS) + (threadIdx.x & 63u);
-                // P0 >= 0: every member has parity P0 at step 0, so step s has parity P0 ^ (s & 1)
-                if (P0 >= 0 && ((s & 1) ^ P0) == 0)
-                    step_cell<ST, LBM_SCHEME_ESOTERIC, COLL, (P0 >= 0 ? 0 : -1), false>(v, ent[lo].pop, ent[lo].pop, a, slot,
-                                                                                 threadIdx.x & 31u, sm[threadIdx.x >> 5]);
-                else if (P0 >= 0)
-                    step_cell<ST, LBM_SCHEME_ESOTERIC, COLL, (P0 >= 0 ? 1 : -1), false>(v, ent[lo].pop, ent[lo].pop, a, slot,
-                                                                                 threadIdx.x & 31u, sm[threadIdx.x >> 5]);
-                else
-                    step_cell<ST, LBM_SCHEME_ESOTERIC, COLL, -1, false>(v, ent[lo].pop, ent[lo].pop, a, slot, threadIdx.x & 31u, sm[threadIdx.x >> 5]);
+                step_cell<ST, LBM_SCHEME_ESOTERIC, COLL, -1, false>(v, ent[lo].pop, ent[lo].pop, a, slot, threadIdx.x & 31u,
+                                                                    sm[threadIdx.x >> 5]);
             }
         }
         if (s + 1 < steps && !grid_barrier(bar, (unsigned int)(s + 1) * gridDim.x, limit_ns)) return;
@@ -2017,16 +2014,16 @@ cudaError_t launch_step_batch_t(const BatchEntry* ent, const int64_t* brick_star
     });
 }
 
-// one cooperative launch of k_step_batch_persistent (128 threads, 8 CTAs per SM at most): as many
+// one cooperative launch of k_step_batch_persistent (128 threads, 6 CTAs per SM): as many
 // CTAs as can be resident, never more than units of work; bar is followed by `steps` ticket
 // counters, all cleared before the launch
-template <int ST, int COLL, int P0>
+template <int ST, int COLL>
 cudaError_t launch_persistent_t(const BatchEntry* ent, const int64_t* brick_start, int n_dom, int64_t total_bricks,
                                 const LevelArgs* args, int steps, GridBarrier* bar, uint64_t limit_ns, cudaStream_t s)
 {
-    constexpr int BRICKS = 2, MINB = 8;
+    constexpr int BRICKS = 2, MINB = 6;
     unsigned int* tickets = reinterpret_cast<unsigned int*>(bar + 1);  // [steps] after the barrier word
-    auto k = k_step_batch_persistent<ST, BRICKS, MINB, COLL, P0>;
+    auto k = k_step_batch_persistent<ST, BRICKS, MINB, COLL>;
     int dev = 0, sms = 0, per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -2041,20 +2038,12 @@ cudaError_t launch_persistent_t(const BatchEntry* ent, const int64_t* brick_star
 
 template <int ST>
 cudaError_t launch_step_batch_persistent(const BatchEntry* ent, const int64_t* brick_start, int n_dom,
-                                         int64_t total_bricks, const LevelArgs* args, int coll, int parity0, int steps,
+                                         int64_t total_bricks, const LevelArgs* args, int coll, int steps,
                                          GridBarrier* bar, uint64_t limit_ns, cudaStream_t s)
 {
     if (total_bricks == 0 || steps == 0) return cudaSuccess;
     return with_coll(coll, [&](auto c) {
-        constexpr int C = decltype(c)::value;
-        // parity-specialised steps for the default rates when the members share a parity
-        if constexpr (C == COLL_CHM_FAST) {
-            if (parity0 == 0)
-                return launch_persistent_t<ST, C, 0>(ent, brick_start, n_dom, total_bricks, args, steps, bar, limit_ns, s);
-            if (parity0 == 1)
-                return launch_persistent_t<ST, C, 1>(ent, brick_start, n_dom, total_bricks, args, steps, bar, limit_ns, s);
-        }
-        return launch_persistent_t<ST, C, -1>(ent, brick_start, n_dom, total_bricks, args, steps, bar, limit_ns, s);
+        return launch_persistent_t<ST, decltype(c)::value>(ent, brick_start, n_dom, total_bricks, args, steps, bar, limit_ns, s);
     });
 }
 

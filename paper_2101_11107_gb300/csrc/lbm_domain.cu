@@ -1282,7 +1282,7 @@ struct lbm_batch {
             if (e == cudaSuccess)
                 e = cudaMemsetAsync(d_bar, 0, sizeof(GridBarrier) + sizeof(unsigned int) * (size_t)steps, stream);
             if (e == cudaSuccess)
-                e = L.step_batch_persistent(d_ent, d_start, n(), total_bricks, d_args, coll, common_parity(0), steps,
+                e = L.step_batch_persistent(d_ent, d_start, n(), total_bricks, d_args, coll, steps,
                                             d_bar, limit_ns, stream);
             if (e == cudaSuccess)
                 e = cudaMemcpyAsync(h_fail, &d_bar->fail, sizeof(unsigned int), cudaMemcpyDeviceToHost, stream);

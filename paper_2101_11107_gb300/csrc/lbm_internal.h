@@ -174,10 +174,9 @@ struct Launchers {
     // storage precision skipped since the last call (0: none; always 0 in the default build)
     unsigned (*debug_fault)();
     // persistent batched step: `steps` steps of every domain in one cooperative launch, a grid
-    // barrier (waits bounded by limit_ns) between steps; args[s][d]; parity0: the parity every
-    // domain has at step 0, or -1
+    // barrier (waits bounded by limit_ns) between steps; args[s][d]
     cudaError_t (*step_batch_persistent)(const BatchEntry* ent, const int64_t* brick_start, int n_dom,
-                                         int64_t total_bricks, const LevelArgs* args, int coll, int parity0, int steps,
+                                         int64_t total_bricks, const LevelArgs* args, int coll, int steps,
                                          GridBarrier* bar, uint64_t limit_ns, cudaStream_t stream);
 };
 // storage-independent output of the running means (lbm_metrics.cu)

@@ -90,3 +90,21 @@ def test_large_domain_gives_the_same_bits(storage):
     assert np.abs(out[0][1]).max() > 0
     for rho, u in out[1:]:
         assert np.array_equal(rho, out[0][0]) and np.array_equal(u, out[0][1])
+
+
+@pytest.mark.parametrize("persistent", [False, True])
+@pytest.mark.parametrize("storage", ["fp32", "fp16"])
+def test_batches_of_porous_boxes(storage, persistent):
+    """The batched kernels run the links in instances of their own: the fields of the boxes stepped alone."""
+    gs = [porous(f, 20 + k) for k, f in enumerate((0.45, 0.8))]
+    doms, alone = ([lbm.Domain.from_geometry(g, storage=storage) for g in gs] for _ in range(2))
+    batch = lbm.Batch(doms, graph_steps=10)
+    batch.set_persistent(persistent)
+    for n in (10, 7, 10):
+        batch.step(n)
+    batch.sync()
+    for d, a in zip(doms, alone):
+        a.step(27)
+        (r1, u1), (r2, u2) = d.macroscopic(), a.macroscopic()
+        assert np.abs(u1).max() > 0 and np.array_equal(r1, r2) and np.array_equal(u1, u2)
+    batch.close()
