@@ -56,12 +56,12 @@ NOMINAL_HBM_GBS = 8000.0  # the metric's roofline denominator (bytes per fluid-c
 K_STEP_TRAFFIC = {
     ("womersley", "fp32", "ab", "256x3"): (120_867_328, "k_step<fp32, A-B, 4 bricks, 3 CTAs/SM, default rates, no links> (89.77 MB read, 31.10 MB written)"),
     ("womersley", "fp32", "ab", "128x7"): (120_340_992, "k_step<fp32, A-B, 2 bricks, 7 CTAs/SM, default rates, no links> (89.81 MB read, 30.53 MB written)"),
-    ("womersley", "fp32", "ab", "128x6"): (119_857_408, "k_step<fp32, A-B, 2 bricks, 8 CTAs/SM, default rates, no links> (89.75 MB read, 30.10 MB written)"),
+    ("womersley", "fp32", "ab", "128x6"): (121_096_704, "k_step<fp32, A-B, 2 bricks, 6 CTAs/SM, default rates, no links> (89.82 MB read, 31.28 MB written)"),
     ("womersley", "fp32", "ab", "128x8"): (120_348_160, "k_step<fp32, A-B, 2 bricks, 8 CTAs/SM, default rates, no links> (89.79 MB read, 30.55 MB written)"),
     ("womersley", "fp32", "ab", "128x10"): (122_133_760, "k_step<fp32, A-B, 2 bricks, 10 CTAs/SM, default rates, no links> (89.72 MB read, 32.42 MB written)"),
     ("womersley", "fp32", "esoteric", "256x3"): (97_949_184, "k_step<fp32, twist, 4 bricks, 3 CTAs/SM, default rates, parity 1, no links> (82.82 MB read, 15.13 MB written)"),
     ("womersley", "fp32", "esoteric", "128x7"): (98_066_432, "k_step<fp32, twist, 2 bricks, 7 CTAs/SM, default rates, parity 1, no links> (82.82 MB read, 15.25 MB written)"),
-    ("womersley", "fp32", "esoteric", "128x6"): (98_080_256, "k_step<fp32, twist, 2 bricks, 8 CTAs/SM, default rates, parity 1, no links> (82.82 MB read, 15.26 MB written)"),
+    ("womersley", "fp32", "esoteric", "128x6"): (97_976_576, "k_step<fp32, twist, 2 bricks, 6 CTAs/SM, default rates, parity 1, no links> (82.83 MB read, 15.14 MB written)"),
     ("womersley", "fp32", "esoteric", "128x8"): (98_131_968, "k_step<fp32, twist, 2 bricks, 8 CTAs/SM, default rates, parity 1, no links> (82.81 MB read, 15.32 MB written)"),
     ("womersley", "fp32", "esoteric", "128x10"): (101_006_080, "k_step<fp32, twist, 2 bricks, 10 CTAs/SM, default rates, parity 1, no links> (82.98 MB read, 18.03 MB written)"),
     ("womersley", "fp32", "esoteric", "pipe128x6"): (95_522_816, "k_step_et_pipe<fp32, 2 bricks, 6 CTAs/SM, persistent> (79.98 MB read, 15.54 MB written)"),
@@ -69,7 +69,7 @@ K_STEP_TRAFFIC = {
     ("womersley", "fp32", "esoteric", "2c128x3"): (97_840_128, "k_step2<fp32, 4 bricks, 3 CTAs/SM> (82.86 MB read, 14.98 MB written)"),
     ("aneurysm512", "fp32", "esoteric", "256x3"): (247_981_312, "k_step<fp32, twist, 4 bricks, 3 CTAs/SM, default rates, parity 1, 3 link rounds> (166.84 MB read, 81.14 MB written)"),
     ("aneurysm512", "fp32", "esoteric", "128x7"): (253_959_424, "k_step<fp32, twist, 2 bricks, 7 CTAs/SM, default rates, parity 1, 3 link rounds> (167.02 MB read, 86.94 MB written)"),
-    ("aneurysm512", "fp32", "esoteric", "128x6"): (248_477_440, "k_step<fp32, twist, 2 bricks, 8 CTAs/SM, default rates, parity 1, 3 link rounds> (166.83 MB read, 81.64 MB written)"),
+    ("aneurysm512", "fp32", "esoteric", "128x6"): (248_123_136, "k_step<fp32, twist, 2 bricks, 6 CTAs/SM, default rates, parity 1, 3 link rounds> (166.84 MB read, 81.28 MB written)"),
     ("aneurysm512", "fp32", "esoteric", "128x8"): (248_439_040, "k_step<fp32, twist, 2 bricks, 8 CTAs/SM, default rates, parity 1, 3 link rounds> (166.81 MB read, 81.63 MB written)"),
     ("aneurysm512", "fp32", "esoteric", "128x10"): (271_365_888, "k_step<fp32, twist, 2 bricks, 10 CTAs/SM, default rates, parity 1, 3 link rounds> (167.36 MB read, 104.01 MB written)"),
     ("aneurysm512", "fp32", "esoteric", "pipe128x6"): (242_021_120, "k_step_et_pipe<fp32, 2 bricks, 6 CTAs/SM, persistent> (159.48 MB read, 82.54 MB written)"),

@@ -221,13 +221,14 @@ lbm_status lbm_get_info(const lbm_domain* dom, lbm_info* out);
 #define LBM_N_LAUNCH_CONFIGS 8
 
 /* Selects the step kernel's launch configuration: 0 = 256 threads (four 4^3 bricks) per CTA
- * with a register budget for 3 resident CTAs per SM; 1, 2, 3, 4 = 128 threads with 7, 6 (8 for a
- * domain of more than 8192 bricks), 8 or 10; 5 = a persistent, software-pipelined variant (128 threads, 6 CTAs per SM; the next cell's
+ * with a register budget for 3 resident CTAs per SM; 1, 2, 3, 4 = 128 threads with 7, 6, 8 or
+ * 10; 5 = a persistent, software-pipelined variant (128 threads, 6 CTAs per SM; the next cell's
  * populations are copied into shared memory asynchronously while the current one is computed;
  * FP32 esoteric twist only, other domains use 3); 6, 7 = two cells per thread (128 threads = four
  * bricks per CTA, 4 or 3 CTAs per SM; the two cells' collisions as packed FP32x2 arithmetic;
  * esoteric twist with CHM-MRT at unit higher-order rates only, other domains use 2).  Results
- * do not depend on it.  Default 2.
+ * do not depend on it.  Default 2; 3 for a domain of more than 8192 bricks, unless it runs the twist
+ * of SRT2 or TRT2 with Bouzidi links (lbm_get_info tells).
  * Errors: INVALID_ARG. */
 lbm_status lbm_set_launch_config(lbm_domain* dom, int32_t config);
 

@@ -989,12 +989,9 @@ __device__ __forceinline__ void gather(const DomainView& v, const void* src, uin
 // ------------------------------------------------------------------------------ kernels
 // Rounds of links a warp holds in registers: six cover every run of the vessels, so no warp of a small
 // domain, whose step is as long as its slowest warp, waits for the reloading loop (25 k cells: 6.5 -> 5.3 us,
-// 150 k: 10.3 -> 9.5 us against three); on a large domain the warps hide one another's latency and the fewer
+// 150 k: 10.3 -> 9.5 us against three); on a large domain (LARGE_BRICKS) the warps hide one another's latency and the fewer
 // registers win (2.7 M cells, 45 k bricks: 124 us with three, 129 us with six; 11 k bricks: 26.0 and 26.9 us).
 constexpr int LINK_ROUNDS = 6, LINK_ROUNDS_LARGE = 3;
-// Bricks from which a domain counts as large here and in the default launch configuration: several waves of
-// CTAs, so that throughput counts and not the slowest warp.
-constexpr int64_t LARGE_BRICKS = 8192;
 
 // Bouzidi links of a warp's cells, shared out among its lanes: the links of a half-brick are one run of the
 // packed list, so a lane takes entry k0 + lane, + 32, ...: code and coefficient (coalesced, before
@@ -1834,20 +1831,19 @@ cudaError_t launch_step_t(const DomainView& v, const void* src, void* dst, const
     return with_coll(a.coll, [&](auto c) {
         constexpr int C = decltype(c)::value;
         constexpr int T = BRICKS * BRICK_CELLS;
-        // the default rates: a domain without Bouzidi cells runs without the link code and its exchange area
-        // (64x64x256 pipe FP16 19.5 us a step, 20.8 us with them), a large one with fewer rounds, and the
-        // twist has one kernel per parity (constant plane indices)
-        if constexpr (C == COLL_CHM_FAST) {
-            constexpr int P0 = SCHEME == LBM_SCHEME_ESOTERIC ? 0 : -1, P1 = SCHEME == LBM_SCHEME_ESOTERIC ? 1 : -1;
-            constexpr int L = LINK_ROUNDS, LL = LINK_ROUNDS_LARGE;
-            const bool large = v.n_bricks > LARGE_BRICKS;
-            auto k = !v.bstart ? (a.parity ? k_step<ST, SCHEME, BRICKS, MINB, C, P1, 0> : k_step<ST, SCHEME, BRICKS, MINB, C, P0, 0>)
-                     : large   ? (a.parity ? k_step<ST, SCHEME, BRICKS, MINB, C, P1, LL> : k_step<ST, SCHEME, BRICKS, MINB, C, P0, LL>)
-                               : (a.parity ? k_step<ST, SCHEME, BRICKS, MINB, C, P1, L> : k_step<ST, SCHEME, BRICKS, MINB, C, P0, L>);
-            return launch_pdl(k, grid, T, 0, s, v, src, dst, a);
-        } else {
-            return launch_pdl(k_step<ST, SCHEME, BRICKS, MINB, C>, grid, T, 0, s, v, src, dst, a);
-        }
+        // The kernel's link rounds: 0 (neither link code nor exchange area) for a domain without Bouzidi cells, where
+        // that is faster: default rates (633 k cell pipe FP16 19.5 us a step, 20.8 us with them), SRT and TRT
+        // on large domains (TRT at 8 CTAs per SM 25.2 and 34.6 us; on 87 k cells 5.4 and 5.1 us), not general
+        // rates (26.4 and 26.0 us); fewer for a large domain with links (2.7 M cells, TRT at 8 CTAs 137 and 152 us).
+        // The twist with the default rates has one kernel per parity (constant plane indices).
+        constexpr bool TWIST = SCHEME == LBM_SCHEME_ESOTERIC, FAST = C == COLL_CHM_FAST;
+        constexpr int P0 = TWIST && FAST ? 0 : -1, P1 = TWIST && FAST ? 1 : -1;
+        constexpr int L = LINK_ROUNDS, LL = LINK_ROUNDS_LARGE, L0 = C == COLL_CHM ? L : 0;
+        const bool large = v.n_bricks > LARGE_BRICKS;
+        auto k = !v.bstart && (FAST || large) ? (a.parity ? k_step<ST, SCHEME, BRICKS, MINB, C, P1, L0> : k_step<ST, SCHEME, BRICKS, MINB, C, P0, L0>)
+                 : v.bstart && large          ? (a.parity ? k_step<ST, SCHEME, BRICKS, MINB, C, P1, LL> : k_step<ST, SCHEME, BRICKS, MINB, C, P0, LL>)
+                                              : (a.parity ? k_step<ST, SCHEME, BRICKS, MINB, C, P1, L> : k_step<ST, SCHEME, BRICKS, MINB, C, P0, L>);
+        return launch_pdl(k, grid, T, 0, s, v, src, dst, a);
     });
 }
 
@@ -1896,11 +1892,7 @@ cudaError_t launch_step_scheme(int config, const DomainView& v, const void* src,
     switch (config) {
     case 0: return launch_step_t<ST, SCHEME, 4, 3>(v, src, dst, a, s);
     case 1: return launch_step_t<ST, SCHEME, 2, 7>(v, src, dst, a, s);
-    // the default: 6 CTAs per SM, 8 on large domains, which the memory system bounds and more loads in flight
-    // help (2.7 M cells FP32 124.6 -> 117.1 us, FP16 105.1 -> 88.7 us; 150 k cells 9.3 -> 9.5 us the other way)
-    case 2:
-        return v.n_bricks > LARGE_BRICKS ? launch_step_t<ST, SCHEME, 2, 8>(v, src, dst, a, s)
-                                         : launch_step_t<ST, SCHEME, 2, 6>(v, src, dst, a, s);
+    case 2: return launch_step_t<ST, SCHEME, 2, 6>(v, src, dst, a, s);
     case 3: return launch_step_t<ST, SCHEME, 2, 8>(v, src, dst, a, s);
     default: return launch_step_t<ST, SCHEME, 2, 10>(v, src, dst, a, s);
     }
@@ -2054,9 +2046,7 @@ cudaError_t launch_step_batch(int config, const BatchEntry* ent, const int64_t* 
     switch (config) {
     case 0: return launch_step_batch_t<ST, 4, 3>(ent, brick_start, n_dom, total_bricks, args, coll, parity, s);
     case 1: return launch_step_batch_t<ST, 2, 7>(ent, brick_start, n_dom, total_bricks, args, coll, parity, s);
-    case 2:  // the default, by size as for a single domain
-        return total_bricks > LARGE_BRICKS ? launch_step_batch_t<ST, 2, 8>(ent, brick_start, n_dom, total_bricks, args, coll, parity, s)
-                                           : launch_step_batch_t<ST, 2, 6>(ent, brick_start, n_dom, total_bricks, args, coll, parity, s);
+    case 2: return launch_step_batch_t<ST, 2, 6>(ent, brick_start, n_dom, total_bricks, args, coll, parity, s);
     case 3: return launch_step_batch_t<ST, 2, 8>(ent, brick_start, n_dom, total_bricks, args, coll, parity, s);
     default: return launch_step_batch_t<ST, 2, 10>(ent, brick_start, n_dom, total_bricks, args, coll, parity, s);
     }

@@ -60,7 +60,7 @@ struct lbm_domain {
     // d_pop[0] holds them in place, arranged for a read of parity time & 1
     int cur = 0;
     void* d_side = nullptr;  // twist: f* of q >= 1/2 Bouzidi links, one entry per packed link
-    int launch_config = DEFAULT_LAUNCH_CONFIG;
+    int chosen_config = -1;  // the launch configuration set or found by autotuning, -1: none yet
     double* d_partials = nullptr;
     lbm_diagnostics* d_diag = nullptr;
     Sum4* d_mean = nullptr;  // running-mean sums (rho, ux, uy, uz) per fluid cell, FP64
@@ -93,6 +93,11 @@ struct lbm_domain {
     bool twist() const { return params.scheme == LBM_SCHEME_ESOTERIC; }
     void* src() const { return d_pop[twist() ? 0 : cur]; }
     void* dst() const { return d_pop[twist() ? 0 : 1 - cur]; }
+    int launch_config() const
+    {
+        return chosen_config >= 0 ? chosen_config
+                                  : default_launch_config(twist(), level_args(0).coll, n_bricks, n_blinks > 0);
+    }
 
     void* dev_alloc(size_t bytes)
     {
@@ -707,10 +712,11 @@ lbm_status lbm_step(lbm_domain* D, int64_t n)
     g_last_error.clear();
     if (!D) return fail(LBM_ERR_INVALID_ARG, "NULL domain");
     if (n < 0) return fail(LBM_ERR_INVALID_ARG, "n must be >= 0");
+    const int config = D->launch_config();
     for (int64_t k = 0; k < n; ++k) {
         const LevelArgs a = D->level_args(D->time);
         cudaError_t e = launchers(D->params.storage)
-                            .step(D->params.scheme, D->launch_config, D->view, D->src(), D->dst(), a, D->stream);
+                            .step(D->params.scheme, config, D->view, D->src(), D->dst(), a, D->stream);
         if (e != cudaSuccess) return cuda_fail(e, "step kernel");
         if (!D->twist()) D->cur = 1 - D->cur;
         D->time += 1;
@@ -723,7 +729,7 @@ lbm_status lbm_set_launch_config(lbm_domain* D, int32_t config)
     g_last_error.clear();
     if (!D) return fail(LBM_ERR_INVALID_ARG, "NULL domain");
     if (config < 0 || config >= N_LAUNCH_CONFIGS) return fail(LBM_ERR_INVALID_ARG, "launch config out of range");
-    D->launch_config = config;
+    D->chosen_config = config;
     return LBM_OK;
 }
 
@@ -743,7 +749,7 @@ lbm_status lbm_autotune(lbm_domain* D, int32_t trial_steps, int32_t* best_config
     g_last_error.clear();
     if (!D || trial_steps < 1) return fail(LBM_ERR_INVALID_ARG, "bad arguments");
     if (D->n_bricks == 0) {
-        if (best_config) *best_config = D->launch_config;
+        if (best_config) *best_config = D->launch_config();
         return LBM_OK;
     }
     // The state is kept: each configuration runs from a copy of the current populations (and
@@ -757,7 +763,7 @@ lbm_status lbm_autotune(lbm_domain* D, int32_t trial_steps, int32_t* best_config
     if (e == cudaSuccess) e = cudaEventCreate(&t0);
     if (e == cudaSuccess) e = cudaEventCreate(&t1);
     const Launchers& L = launchers(D->params.storage);
-    int best = D->launch_config;
+    int best = D->launch_config();
     float best_ms = INFINITY;
     for (int c = 0; c < N_LAUNCH_CONFIGS && e == cudaSuccess; ++c) {
         if (!config_applies(D, c)) {
@@ -796,7 +802,7 @@ lbm_status lbm_autotune(lbm_domain* D, int32_t trial_steps, int32_t* best_config
     if (t1) cudaEventDestroy(t1);
     D->dev_free(keep, pb + sb);
     if (e != cudaSuccess) return cuda_fail(e, "autotune");
-    D->launch_config = best;
+    D->chosen_config = best;
     if (best_config) *best_config = best;
     return LBM_OK;
 }
@@ -1033,7 +1039,7 @@ lbm_status lbm_get_info(const lbm_domain* D, lbm_info* out)
     I.storage = D->params.storage;
     I.bytes_per_value = D->bytes_per_value();
     I.device_bytes = D->device_bytes;
-    I.launch_config = D->launch_config;
+    I.launch_config = D->launch_config();
     I.scheme = D->params.scheme;
     I.n_store_bricks = D->n_store_bricks;
     I.n_halo = D->n_halo;
@@ -1214,7 +1220,7 @@ struct lbm_batch {
     std::vector<lbm_domain*> doms;
     int storage = 0;
     int coll = COLL_CHM_FAST;
-    int launch_config = DEFAULT_LAUNCH_CONFIG;
+    int launch_config = DEFAULT_BATCH_CONFIG;
     int graph_steps = 0;
     int64_t total_bricks = 0, total_fluid = 0;
     cudaStream_t stream = nullptr;       // private non-blocking stream: work and graph capture

@@ -141,7 +141,22 @@ constexpr int N_LAUNCH_CONFIGS = 8;
 
 // collision kernels (the `coll` of LevelArgs and the COLL template parameter of the step kernels)
 constexpr int COLL_CHM = 0, COLL_CHM_FAST = 1, COLL_SRT2 = 2, COLL_TRT2 = 3;
-constexpr int DEFAULT_LAUNCH_CONFIG = 2;  // 128 threads, 6 CTAs per SM
+// Bricks from which a domain counts as large, in the kernels' link rounds and in the default configuration:
+// several waves of CTAs, so that throughput counts and not the slowest warp.
+constexpr int64_t LARGE_BRICKS = 8192;
+// The launch configuration of a domain until one is set: 128 threads with 6 CTAs per SM (2), on large domains 8
+// (3), which the memory system bounds and more loads in flight help.  6 and 8 CTAs, us a step: 150 k cells FP32
+// 9.3 and 9.5; 2.7 M cells with links (45 k bricks): default rates FP32 124.6 and 117.1, general rates 129.4
+// and 120.5, A-B TRT 127.6 and 118.0; 2.7 M cells without, TRT 124.7 and 116.4.  The twist of SRT and TRT with
+// links does not fit 64 registers and keeps 6: TRT 129.2 and 137.3 us at 45 k bricks, 30.0 and 33.1 us at 13 k.
+constexpr int default_launch_config(bool twist, int coll, int64_t n_bricks, bool links)
+{
+    const bool tight = twist && links && (coll == COLL_SRT2 || coll == COLL_TRT2);
+    return n_bricks > LARGE_BRICKS && !tight ? 3 : 2;
+}
+// ... and of a batch: its kernel has six link rounds at every size.  6 and 8 CTAs, FP32 default rates: 12 k bricks
+// 23.6 and 25.6 us a step, 36 k bricks 85.1 and 88.8 us; TRT 30.8 and 37.9, 103 and 117 us.
+constexpr int DEFAULT_BATCH_CONFIG = 2;
 
 // Launchers, one set per storage precision (lbm_step_<storage>.cu).  All enqueue on `stream`
 // and return the launch status.

@@ -2,6 +2,8 @@
 box drives that at its edges: half-bricks with no link, a few, and several hundred (more rounds than a
 warp holds in registers), cells walled on both sides of a direction, wall links without a q, q on both
 sides of 1/2 and exactly 1/2."""
+import dataclasses
+import functools
 import os
 
 import numpy as np
@@ -108,3 +110,45 @@ def test_batches_of_porous_boxes(storage, persistent):
         (r1, u1), (r2, u2) = d.macroscopic(), a.macroscopic()
         assert np.abs(u1).max() > 0 and np.array_equal(r1, r2) and np.array_equal(u1, u2)
     batch.close()
+
+
+@pytest.mark.parametrize("persistent", [False, True])
+def test_batch_of_more_than_8192_bricks(persistent):
+    gs = [porous(0.6, 30, shape=(64, 84, 64)), porous(0.99, 31, shape=(64, 64, 64))]
+    doms, alone = ([lbm.Domain.from_geometry(g) for g in gs] for _ in range(2))
+    assert sum(d.info()["n_bricks"] for d in doms) > 8192
+    batch = lbm.Batch(doms, graph_steps=4)
+    batch.set_persistent(persistent)
+    batch.step(11)
+    batch.sync()
+    for d, a in zip(doms, alone):
+        a.step(11)
+        (r1, u1), (r2, u2) = d.macroscopic(dense=False), a.macroscopic(dense=False)
+        assert np.abs(u1).max() > 0 and np.array_equal(r1, r2) and np.array_equal(u1, u2)
+    batch.close()
+
+
+@functools.lru_cache(maxsize=1)
+def _large_box():
+    return porous(0.6, 14, shape=(64, 84, 128))
+
+
+@pytest.mark.parametrize("storage", ["fp32", "bf16"])
+@pytest.mark.parametrize("collision", ["srt2", "trt2"])
+@pytest.mark.parametrize("bouzidi", [True, False])
+def test_large_domain_of_the_other_operators(bouzidi, collision, storage):
+    """Their kernels without links and with three rounds, against the pipelined one and A-B, bit for bit."""
+    g = _large_box()
+    if not bouzidi:
+        g = dataclasses.replace(g, links=None)
+    out = []
+    for scheme, configs in (("esoteric", (0, 1, 2, 3, 4, 5)), ("ab", (2, 3))):
+        for config in configs:
+            d = lbm.Domain.from_geometry(g, scheme=scheme, storage=storage, collision=collision)
+            d.set_launch_config(config)
+            d.step(7)
+            out.append(d.macroscopic(dense=False))
+            d.close()
+    assert np.abs(out[0][1]).max() > 0
+    for rho, u in out[1:]:
+        assert np.array_equal(rho, out[0][0]) and np.array_equal(u, out[0][1])

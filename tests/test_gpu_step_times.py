@@ -46,6 +46,40 @@ def test_16_bit_ab_step_is_no_slower_than_fp32(large_pipe, collision, storage):
     assert t[storage] <= 1.05 * t["fp32"], t
 
 
+@pytest.mark.parametrize("scheme", ["esoteric", "ab"])
+@pytest.mark.parametrize("case", ["default", "rates", "srt2", "trt2"])
+def test_default_configuration_is_a_fast_one(large_pipe, case, scheme):
+    """The configuration that a large domain starts with is within 8% of the best of the one-cell kernels."""
+    kw = dict(default={}, rates=dict(omega_hi=(1.2, 1.1, 1.05, 0.95))).get(case, dict(collision=case))
+    d = lbm.Domain.from_geometry(large_pipe, scheme=scheme, **kw)
+    first = d.info()["launch_config"]
+    t = gpu_us(lambda: d.step(40), 40)
+    times = {}
+    for c in range(5):
+        d.set_launch_config(c)
+        assert d.info()["launch_config"] == c
+        times[lbm.LAUNCH_CONFIG_NAMES[c]] = gpu_us(lambda: d.step(40), 40)
+    d.close()
+    assert t <= 1.08 * min(times.values()), (lbm.LAUNCH_CONFIG_NAMES[first], t, times)
+    # the name is that of the kernel that runs
+    assert abs(t - times[lbm.LAUNCH_CONFIG_NAMES[first]]) <= 0.05 * t, (lbm.LAUNCH_CONFIG_NAMES[first], t, times)
+
+
+def test_default_configuration_by_size():
+    """6 CTAs per SM up to 8192 bricks; 8 above, but for the twist of TRT2 with links."""
+    small = I.pipe(32, 32, 64, 12.0, tau=0.6, g0=(0.0, 0.0, 1e-6))
+    large = I.pipe(64, 64, 256, 28.0, tau=0.6, g0=(0.0, 0.0, 1e-6))
+    linked = I.pipe(64, 64, 256, 28.0, tau=0.6, g0=(0.0, 0.0, 1e-6), bouzidi=True)
+    for g, kw, want in ((small, {}, "128x6"), (large, {}, "128x8"), (large, dict(collision="trt2"), "128x8"),
+                        (linked, {}, "128x8"), (linked, dict(collision="trt2"), "128x6"),
+                        (linked, dict(collision="trt2", scheme="ab"), "128x8")):
+        d = lbm.Domain.from_geometry(g, **kw)
+        assert lbm.LAUNCH_CONFIG_NAMES[d.info()["launch_config"]] == want
+        d.set_launch_config(2)
+        assert d.info()["launch_config"] == 2
+        d.close()
+
+
 @pytest.mark.parametrize("storage", ["fp32", "fp16"])
 def test_persistent_batch_with_default_rates_is_the_fastest(storage):
     """The default rates leave out the higher moments, which general rates compute on top (5% for the spread of
