@@ -268,14 +268,20 @@ __device__ __forceinline__ uint32_t ab_offset_shfl(uint32_t n, int32_t row_lane,
     return ((wm >> i) & 1u) ? (uint32_t)(Q - 1 - i) * n + slot : (uint32_t)i * n + s;
 }
 
-// Whether an A-B step forms all its offsets before its first load.  Loads are plain (a step may start while the
-// one before it still writes) and stay in order with the shuffles, and a shuffle between two loads waits
-// for the loads before it: few are in flight at a time.  Per step, one by one -> all first: 2.7 M cell Bouzidi
-// pipe FP16 170 -> 98 us, FP16 TRT 197 -> 108 us, FP32 TRT 124 -> 118 us; 633 k cell pipe FP16 TRT 43.4 -> 25.3 us,
-// FP32 TRT 31.9 -> 29.0 us.  FP32 with the default rates keeps them one by one: 109 us, and 116 us all first
-// (2.7 M cells); 26.8 and 26.9 us (633 k cells).
-template <int ST, int COLL>
-__host__ __device__ constexpr bool ab_offsets_first() { return !(ST == LBM_STORE_FP32 && COLL == COLL_CHM_FAST); }
+// How many offsets an A-B step forms before it loads from them.  Loads are plain (a step may start while the one
+// before it still writes) and stay in order with the shuffles, and a shuffle waits for the loads before it, so
+// between groups few loads are in flight.  All 27 in one group is the fastest but for the default rates in FP32
+// (one by one) and in 16 bits without links (three).  us a step, one by one / threes / all:
+//   2.7 M cell Bouzidi pipe  FP16 170 / 149 / 98    FP16 TRT 197 / - / 108    FP32 TRT 124 / - / 118
+//   633 k cell pipe          FP16 22.3 / 21.9 / 20.8    FP16 TRT 43.5 / - / 25.0
+//   95 k cell pipe           FP16 5.4 / 5.4 / 6.2
+//   FP32, default rates: 2.7 M cells 109 / 109 / 116, 95 k cells 4.6 / 4.9 / 6.1
+template <int ST, int COLL, int LINKS>
+__host__ __device__ constexpr int ab_group()
+{
+    if (COLL != COLL_CHM_FAST) return Q;
+    return ST == LBM_STORE_FP32 ? 1 : LINKS == 0 ? 3 : Q;
+}
 
 // Twist corner slots in the step kernel: lanes hold the brick's nb8 row (lane & 7).
 __device__ __forceinline__ void corner_slots_shfl(int32_t row_lane, uint32_t slot, uint32_t (&cs)[8])
@@ -1168,20 +1174,24 @@ __device__ __forceinline__ void step_cell(const DomainView& v, const void* src, 
         if (fluid) fetch_et<ST, PC>(dst, n, cs, wm, a.parity, d, clean);
     } else {
         const int32_t row = __ldg(v.nbr + brick * (uint32_t)Q + (lane < (uint32_t)Q ? lane : 0u));
-        constexpr bool FIRST = ab_offsets_first<ST, COLL>();
+        constexpr int G = ab_group<ST, COLL, LINKS>();
         uint32_t off[Q];
-        if (FIRST)
+        if (G == Q)
 #pragma unroll
             for (int i = 0; i < Q; ++i) off[i] = ab_offset_shfl(n, row, slot, wm, i);
         if (LINKS) links.prefetch(v);
         if (PDL) pdl_wait();
-        if (FIRST) {
+        if (G == Q) {
             if (fluid) fetch_ab_at<ST>(src, n, off, d);
         } else {
 #pragma unroll
-            for (int i = 0; i < Q; ++i) {
-                off[i] = ab_offset_shfl(n, row, slot, wm, i);
-                if (fluid) d[i] = LBM_IN_RANGE(off[i], (uint64_t)Q * n, 1) ? Store<ST>::load_rw_h(src, off[i]) : 0.0f;
+            for (int g = 0; g < Q; g += G) {
+#pragma unroll
+                for (int j = 0; j < G; ++j) off[g + j] = ab_offset_shfl(n, row, slot, wm, g + j);
+                if (fluid)
+#pragma unroll
+                    for (int j = 0; j < G; ++j)
+                        d[g + j] = LBM_IN_RANGE(off[g + j], (uint64_t)Q * n, 1) ? Store<ST>::load_rw_h(src, off[g + j]) : 0.0f;
             }
             if (fluid) scale_in<ST>(d);
         }
