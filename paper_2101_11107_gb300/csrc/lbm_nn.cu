@@ -726,12 +726,12 @@ __global__ void k_prepare(const float* __restrict__ master, __nv_bfloat16* __res
 
 // coarse (X,Y,Z) = mean of rho and u over the fluid fine children (2X+a, 2Y+b, 2Z+c); 0 if none.  A thread
 // takes W consecutive coarse cells of a row: with W = 4 the mask comes as four 8-byte words, most of
-// which are 0 (a vessel fills about 2% of its box), and the four planes go out as 16-byte stores, so
-// the kernel moves the mask and the coarse fields at memory speed; the fluid children are read one by
-// one, in the order of the sum (z, y, x), whatever W is.  W = 1: rows or arrays that the wide
-// accesses do not fit.  256^3 -> 128^3 vessel, ncu: 26.2 us with one cell
-// a thread, 16.7 us with four (22 MB read, 34 MB written).
-template <int W>
+// which are 0 (a vessel fills about 2% of its box), and the four planes go out as 16-byte stores.  WIDE: the
+// fields of eight fine cells in a row come as two 16-byte words each, wherever one of them is fluid (one sector,
+// which a single cell would fetch too); else the fluid children one by one.  The sum runs in the order z, y, x
+// in every form.  What bounds it is memory traffic; us at 256^3 -> 128^3, one cell a thread / four / four and wide:
+// vessel 24.8 / 11.1 / 10.3, one cell in fifty 39 / 54 / 37, all cells 52 / 99 / 52 (319 MB: 6.2 TB/s).
+template <int W, bool WIDE>
 __global__ void __launch_bounds__(256)
     k_restrict(const float* __restrict__ frho, const float* __restrict__ fu, const uint8_t* __restrict__ fmask, int fnx,
                int fny, int fnz, float* __restrict__ crho, float* __restrict__ cu)
@@ -744,44 +744,62 @@ __global__ void __launch_bounds__(256)
     const int X = (int)(c - (int64_t)row * cnx), Y = (int)(row % (uint32_t)cny), Z = (int)(row / (uint32_t)cny);
     uint8_t m[4][2 * W];
     int64_t at[4];
-    bool any = false;
+    bool any[4];
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
         at[r] = 2 * X + (int64_t)fnx * ((2 * Y + (r & 1)) + (int64_t)fny * (2 * Z + (r >> 1)));
         if constexpr (W == 4) {
             const uint2 v = __ldg(reinterpret_cast<const uint2*>(fmask + at[r]));
             memcpy(m[r], &v, 8);
-            any = any || (v.x | v.y);
+            any[r] = (v.x | v.y) != 0;
         } else {
+            any[r] = false;
 #pragma unroll
             for (int x = 0; x < 2 * W; ++x) {
                 m[r][x] = fmask[at[r] + x];
-                any = any || m[r][x];
+                any[r] = any[r] || m[r][x];
             }
         }
     }
     float o[4][W] = {};
-    if (any) {
+    int k[W] = {};
+    if constexpr (WIDE) {
 #pragma unroll
-        for (int w = 0; w < W; ++w) {
-            float s[4] = {0.f, 0.f, 0.f, 0.f};
-            int k = 0;
+        for (int r = 0; r < 4; ++r) {
+            if (!any[r]) continue;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float4* f = reinterpret_cast<const float4*>((q ? fu + (q - 1) * fn : frho) + at[r]);
+                const float4 a = __ldg(f), b = __ldg(f + 1);
+                const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+                for (int x = 0; x < 8; ++x)
+                    if (m[r][x]) o[q][x / 2] += v[x];
+            }
+#pragma unroll
+            for (int x = 0; x < 8; ++x) k[x / 2] += m[r][x] != 0;
+        }
+    } else if (any[0] || any[1] || any[2] || any[3]) {
+#pragma unroll
+        for (int w = 0; w < W; ++w)
 #pragma unroll
             for (int r = 0; r < 4; ++r)
 #pragma unroll
                 for (int x = 0; x < 2; ++x) {
                     if (!m[r][2 * w + x]) continue;
                     const int64_t f = at[r] + 2 * w + x;
-                    ++k;
-                    s[0] += frho[f];
-                    s[1] += fu[f];
-                    s[2] += fu[fn + f];
-                    s[3] += fu[2 * fn + f];
+                    ++k[w];
+                    o[0][w] += frho[f];
+                    o[1][w] += fu[f];
+                    o[2][w] += fu[fn + f];
+                    o[3][w] += fu[2 * fn + f];
                 }
-            const float inv = k ? 1.0f / (float)k : 0.0f;
+    }
 #pragma unroll
-            for (int q = 0; q < 4; ++q) o[q][w] = s[q] * inv;
-        }
+    for (int w = 0; w < W; ++w) {
+        const float inv = k[w] ? 1.0f / (float)k[w] : 0.0f;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) o[q][w] *= inv;
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -1218,13 +1236,13 @@ lbm_status lbm_restrict(const float* fine_rho, const float* fine_u, const uint8_
         return nn_fail(LBM_ERR_INVALID_ARG, "fine extents must be positive and even");
     const int64_t cn = (int64_t)(fnx / 2) * (fny / 2) * (fnz / 2);
     const cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    // rows of whole groups of four coarse cells, and arrays on the boundaries of the wide accesses
-    const bool wide = fnx % 8 == 0 && (reinterpret_cast<uintptr_t>(fine_mask) & 7u) == 0 &&
-                      ((reinterpret_cast<uintptr_t>(coarse_rho) | reinterpret_cast<uintptr_t>(coarse_u)) & 15u) == 0;
-    if (wide)
-        k_restrict<4><<<blocks(cn / 4, 256), 256, 0, st>>>(fine_rho, fine_u, fine_mask, fnx, fny, fnz, coarse_rho, coarse_u);
-    else
-        k_restrict<1><<<blocks(cn, 256), 256, 0, st>>>(fine_rho, fine_u, fine_mask, fnx, fny, fnz, coarse_rho, coarse_u);
+    // four cells a thread: rows of whole groups, arrays on the boundaries of the wide accesses, and enough groups for
+    // the chip (128^3 -> 64^3: vessel 6.5 us with four and 4.5 with one, all cells 8.1 and 6.5; 144^3: 6.3 and 8.4)
+    const auto aligned = [](const void* p, uintptr_t n) { return reinterpret_cast<uintptr_t>(p) % n == 0; };
+    const bool four = cn > (1 << 18) && fnx % 8 == 0 && aligned(fine_mask, 8) && aligned(coarse_rho, 16) && aligned(coarse_u, 16);
+    const bool wide = four && aligned(fine_rho, 16) && aligned(fine_u, 16);
+    auto k = wide ? k_restrict<4, true> : four ? k_restrict<4, false> : k_restrict<1, false>;
+    k<<<blocks(four ? cn / 4 : cn, 256), 256, 0, st>>>(fine_rho, fine_u, fine_mask, fnx, fny, fnz, coarse_rho, coarse_u);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return nn_fail(LBM_ERR_CUDA, std::string("restrict: ") + cudaGetErrorString(e));
     return LBM_OK;

@@ -70,3 +70,25 @@ def test_forward_clears_the_box(offset):
     du = du.reshape(want.shape)
     assert torch.equal(du, want) and float(want.abs().max()) > 0
     assert not bool(du[:, fluid == 0].any())
+
+
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("fill", [0.03, 0.6, 1.0])
+def test_restrict_large_enough_for_four_cells_a_thread(fill, offset):
+    """The wide form, and with fields off the 16-byte boundary the form that reads the children one by one; what
+    solid cells hold is not read into a sum."""
+    shape = (66, 178, 192)  # 281,952 coarse cells, rows of whole groups
+    rng = torch.Generator("cuda").manual_seed(3)
+    m = (torch.rand(shape, device="cuda", generator=rng) < fill).to(torch.uint8)
+    f = torch.randn((4, *shape), device="cuda", generator=rng)
+    nan = torch.where(m.bool(), f, torch.full_like(f, float("nan")))
+    rho, u = _at(m.numel(), torch.float32, offset), _at(3 * m.numel(), torch.float32, offset)
+    rho.copy_(nan[0].reshape(-1))
+    u.copy_(nan[1:].reshape(-1))
+    crho, cu = lbm.restrict(rho.reshape(shape), u.reshape(3, *shape), m)
+    split = lambda t: t.double().reshape(33, 2, 89, 2, 96, 2)  # noqa: E731
+    k = split(m).sum((1, 3, 5))
+    for q, got in enumerate([crho, *cu]):
+        v = split(f[q] * m)
+        bound = 9 * 2.0 ** -24 * v.abs().sum((1, 3, 5)) + 1e-30  # as above
+        assert bool(((got.double() - v.sum((1, 3, 5)) / k.clamp(min=1)).abs() <= bound).all())

@@ -96,3 +96,14 @@ def test_persistent_batch_with_default_rates_is_the_fastest(storage):
         for d in doms:
             d.close()
     assert t[(1.0, 1.0, 1.0, 1.0)] <= 1.05 * t[(1.2, 1.1, 1.05, 0.95)], t
+
+
+def test_restriction_of_a_full_box_is_no_slower_than_a_copy():
+    """It reads the fine fields and a mask byte per cell and writes an eighth: 0.6 of a copy's bytes."""
+    n = 256
+    rho, u = torch.rand((n, n, n), device="cuda"), torch.rand((3, n, n, n), device="cuda")
+    mask = torch.ones((n, n, n), dtype=torch.uint8, device="cuda")
+    rho2, u2 = torch.empty_like(rho), torch.empty_like(u)
+    t = gpu_us(lambda: [lbm.restrict(rho, u, mask) for _ in range(10)], 10)
+    copy = gpu_us(lambda: [(rho2.copy_(rho), u2.copy_(u)) for _ in range(10)], 10)
+    assert t <= copy, (t, copy)
