@@ -107,3 +107,20 @@ def test_restriction_of_a_full_box_is_no_slower_than_a_copy():
     t = gpu_us(lambda: [lbm.restrict(rho, u, mask) for _ in range(10)], 10)
     copy = gpu_us(lambda: [(rho2.copy_(rho), u2.copy_(u)) for _ in range(10)], 10)
     assert t <= copy, (t, copy)
+
+
+def test_forward_on_a_nearly_empty_box_costs_its_clear():
+    """One tile of fluid in a 256^3 box: the pass on a small box with the same tile, and a clear of the correction
+    (1.5 for the spread and the clear's own launch)."""
+    def forward(n):
+        mask = np.zeros((n, n, n), np.uint8)
+        mask[n // 2:n // 2 + 4, n // 2:n // 2 + 4, n // 2:n // 2 + 4] = 1
+        net = lbm.Corrector(mask, I.corrector_init_params(1), 0.05, 0.01, 0.005)
+        rho, u = torch.ones(mask.shape, device="cuda"), torch.zeros((3, *mask.shape), device="cuda")
+        t = gpu_us(lambda: [net.forward(rho, u) for _ in range(10)], 10)
+        clear = gpu_us(lambda: [u.zero_() for _ in range(10)], 10)
+        net.close()
+        return t, clear
+
+    (small, _), (large, clear) = forward(64), forward(256)
+    assert large <= 1.5 * (small + clear), (small, large, clear)
