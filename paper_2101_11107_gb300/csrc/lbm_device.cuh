@@ -1828,7 +1828,9 @@ cudaError_t launch_pdl(void (*k)(P...), int grid, int block, size_t smem, cudaSt
     c.stream = s;
     c.attrs = &at;
     c.numAttrs = 1;
-    return cudaLaunchKernelEx(&c, k, P(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&c, k, P(args)...);
+    if (e != cudaSuccess) cudaGetLastError();  // reported here: a later launch that asks must not find it again
+    return e;
 }
 
 // Launch configurations of the step kernel: (bricks per CTA, minimum resident CTAs per SM);

@@ -132,7 +132,9 @@ cudaError_t launch_pdl(void (*k)(P...), dim3 grid, int block, size_t smem, cudaS
     c.stream = s;
     c.attrs = &at;
     c.numAttrs = 1;
-    return cudaLaunchKernelEx(&c, k, P(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&c, k, P(args)...);
+    if (e != cudaSuccess) cudaGetLastError();  // reported here: a later launch that asks must not find it again
+    return e;
 }
 
 __device__ __forceinline__ uint32_t su32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -935,8 +937,8 @@ struct lbm_corrector {
     }
     // Whether the features kernel, one CTA a slab, clears the correction box on its way, which saves a launch (us a
     // forward pass: 128^3 vessel 45.4 -> 37.1, 256^3 vessel 113.1 -> 109.4).  With few slabs in a large box, or words
-    // of 4 bytes in one, a clear by itself is faster: 256^3 with 24 slabs 53.5 us, 112.6 in the kernel; with 72, 54.7 and
-    // 58.4; with 216 (78 k cells a slab), 60.9 and 53.2; 256^3 vessel off the 16-byte boundary 117.2 and 130.9.
+    // of 4 bytes in one, a clear by itself is faster: 256^3 with 24 slabs 45.5 us, 112.3 in the kernel; with 72, 46.0 and
+    // 58.0; with 216 (78 k cells a slab), 51.8 and 51.4; 256^3 vessel off the 16-byte boundary 111.1 and 130.6.
     bool features_clear(const float* du) const
     {
         return n_cells <= ((int64_t)1 << 17) * n_slabs &&

@@ -182,3 +182,28 @@ def test_corrector_fallback_to_plain_solver():
     twin.step(40)
     assert dom.diagnostics()["n_nonfinite"] == 0
     assert all(np.array_equal(x, y) for x, y in zip(dom.macroscopic(), twin.macroscopic()))
+
+
+@pytest.mark.parametrize("scheme", ["esoteric", "ab"])
+def test_a_refused_launch_does_not_fail_the_next_call(scheme):
+    """A step on a stream whose capture has become invalid is refused by the runtime, on the host.  Once the capture
+    has ended, the calls after it work: the refused launch's error code is not found again by a later one."""
+    cu = ctypes.CDLL("libcuda.so.1")
+    g = I.pipe(20, 20, 16, 8.0, tau=0.6, g0=(0.0, 0.0, 1e-5), bouzidi=True)
+    s = torch.cuda.Stream()
+    a = lbm.Domain.from_geometry(g, scheme=scheme, stream=s)
+    b = lbm.Domain.from_geometry(g, scheme=scheme)
+    rho, u = torch.ones(g.mask.shape, device="cuda"), torch.zeros((3, *g.mask.shape), device="cuda")
+    torch.cuda.synchronize()
+    stream, graph = ctypes.c_void_p(s.cuda_stream), ctypes.c_void_p()
+    assert cu.cuStreamBeginCapture_v2(stream, 1) == 0
+    assert cu.cuStreamSynchronize(stream) != 0  # not allowed in a capture: it becomes invalid
+    with pytest.raises(lbm.LbmError):
+        a.step(1)
+    assert cu.cuStreamEndCapture(stream, ctypes.byref(graph)) != 0 and not graph.value
+    assert a.time == 0
+    for d in (a, b):
+        d.init_equilibrium(rho, u)
+        d.step(9)
+    (r1, u1), (r2, u2) = a.macroscopic(), b.macroscopic()
+    assert np.abs(u1).max() > 0 and np.array_equal(r1, r2) and np.array_equal(u1, u2)
