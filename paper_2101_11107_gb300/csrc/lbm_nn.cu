@@ -92,6 +92,7 @@ constexpr uint32_t W_OFF = 2 * HALO_BYTES;              // weights after the two
 constexpr uint32_t W_BYTES = 27 * 512;                  // one layer's weights, BF16
 constexpr uint32_t CONV_SMEM = W_OFF + W_BYTES;         // 48640 B
 constexpr int CONV_CTAS_PER_SM = 4;
+constexpr uint32_t CONV_COLS = 64;  // tensor-memory columns of a CTA
 constexpr int TC_WAIT_LIMIT = 1 << 22;
 
 // Programmatic dependent launch along a pass's chain of kernels (features, then convolutions, loss, weight
@@ -194,7 +195,8 @@ __global__ void __launch_bounds__(128)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {  // two accumulators of 16 columns, at columns 0 and 32
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 64;" ::"r"(su32(&tmem_base))
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&tmem_base)),
+                     "n"(CONV_COLS)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -349,7 +351,7 @@ __global__ void __launch_bounds__(128)
         }
     }
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 64;" ::"r"(tbase) : "memory");
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tbase), "n"(CONV_COLS) : "memory");
 }
 
 // Partial weight gradient of this CTA's slabs on the 5th-generation tensor cores:
@@ -375,10 +377,23 @@ constexpr uint32_t WG_A = (WG_HROWS + 2) * WG_ROW;     // + 2 rows read only by 
 constexpr uint32_t WG_B = SL_Y * 256;                  // dy of the slab: 16 x rows of [co][8 cells]
 constexpr uint32_t WG_BUF = WG_A + WG_B;               // 47104
 constexpr uint32_t WG_SMEM = 2 * WG_BUF;               // 94208
+constexpr uint32_t WG_COLS = 256;                      // tensor-memory columns of a CTA
 // furthest byte an MMA reads in a buffer: A of the last offset pair's last K step
 static_assert((uint32_t)(((HZ - 1) * HY + (SL_Y - 2) + 2) * WG_ROW) + WG_ROW + 15 * 128 + 128 <= WG_A,
               "weight-gradient A operand reads past its buffer");
 static_assert((SL_Y - 2) * 256 + 256 + 128 + 128 <= (int)WG_B, "weight-gradient B operand reads past its buffer");
+
+// A convolution lets the next kernel start before its own CTAs have allocated their tensor memory, and the next one's
+// CTAs hold theirs while they wait for it.  An allocation must therefore never need columns of a CTA that waits:
+// whatever set of these CTAs fits on an SM by shared memory (228 KB, 1 KB of it reserved per CTA) also fits by columns.
+constexpr bool tmem_fits()
+{
+    for (uint32_t w = 0; w <= 2; ++w)
+        for (uint32_t c = 0; c <= 8; ++c)
+            if (w * (WG_SMEM + 1024) + c * (CONV_SMEM + 1024) <= 228u * 1024 && w * WG_COLS + c * CONV_COLS > 512) return false;
+    return 3 * (WG_SMEM + 1024) > 228u * 1024;
+}
+static_assert(tmem_fits(), "CTAs of overlapping kernels could wait for one another's tensor memory");
 
 // The three layers run in one launch (blockIdx.y: the layer), so one layer's tail fills with the next
 // one's CTAs: the three weight gradients depend on nothing but the back-propagated gradients.
@@ -405,7 +420,8 @@ __global__ void __launch_bounds__(128)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {  // nine accumulators of 16 columns at columns 0, 16, ..., 128
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;" ::"r"(su32(&tmem_base))
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&tmem_base)),
+                     "n"(WG_COLS)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -560,7 +576,7 @@ __global__ void __launch_bounds__(128)
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tbase) : "memory");
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tbase), "n"(WG_COLS) : "memory");
 }
 
 // Position of weight (o, co, ci) in a layer's BF16 block, which is the convolution's shared-memory

@@ -1,5 +1,7 @@
 """Consecutive steps overlap on the stream (a step starts while the one before it drains): the
 fields must be those of steps that are waited for one by one, and of captured steps replayed."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -67,3 +69,25 @@ def test_batch_chunks_in_flight(graph_steps):
         (r1, u1), (r2, u2) = d.macroscopic(), a.macroscopic()
         assert np.abs(u1).max() > 0 and np.array_equal(r1, r2) and np.array_equal(u1, u2)
     batch.close()
+
+
+def test_queued_training_steps_equal_waited_ones():
+    """Training steps without a loss are only enqueued: each one's weight update has to be seen by the weight copies
+    of the next one's convolutions, which run ahead of the kernels before them."""
+    g = I.aneurysm(5, edge=64)
+    mask = (g.mask > 0).astype(np.uint8)
+    fluid = torch.from_numpy(mask).cuda()
+    gen = torch.Generator("cuda").manual_seed(2)
+    rho = 1.0 + 0.01 * torch.randn(mask.shape, device="cuda", generator=gen) * fluid
+    u, target = (0.03 * torch.randn((3, *mask.shape), device="cuda", generator=gen) * fluid for _ in range(2))
+    nets = [lbm.Corrector(mask, I.corrector_init_params(4), 0.05, 0.01, 0.005) for _ in range(2)]
+    p = lambda t: ctypes.c_void_p(t.data_ptr())  # noqa: E731
+    for _ in range(12):
+        assert lbm.load_library().lbm_corrector_train_step(nets[0]._h, None, None, p(rho), p(u), p(target), 1e-3, None) == 0
+    for _ in range(12):
+        nets[1].train_step(rho, u, target, 1e-3)
+        torch.cuda.synchronize()
+    queued, waited = (n.params() for n in nets)
+    assert np.abs(waited - lbm.flatten_params(I.corrector_init_params(4))).max() > 1e-3
+    assert np.array_equal(queued, waited)
+    assert torch.equal(nets[0].forward(rho, u), nets[1].forward(rho, u))
