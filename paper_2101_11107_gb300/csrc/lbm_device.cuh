@@ -1226,21 +1226,22 @@ __device__ __forceinline__ void step_cell(const DomainView& v, const void* src, 
     }
 }
 
-// The block's place in the sweep over the bricks.  Where the state outgrows L2, odd levels sweep backwards: a
-// step then begins with the bricks that the step before it touched last, which L2 still holds; in one fixed
-// order such a state evicts itself before it comes round again.  Per step, twist: 2.7 M cell pipe FP32 (337 MB)
-// 117.5 -> 110.4 us, FP16 (168 MB) 89.3 -> 84.5 us; A-B: 633 k cell pipe FP32 (152 MB) 27.9 -> 26.9 us, FP16 (76 MB)
-// 23.0 -> 22.2 us.  At 44 MB and less, all of it in L2, one order is as good or better (19.4 and 19.5 us), and so it
-// is for two arrays far larger than L2 (A-B, 2.7 M cells: FP32, 673 MB, 110 us both ways; FP16, 337 MB, 147 and
-// 171 us).
-constexpr int64_t SWEEP_BYTES = (int64_t)64 << 20, SWEEP_BYTES_AB = (int64_t)256 << 20;
+// The block's place in the sweep over the bricks.  Where the state outgrows what L2 keeps, odd levels sweep backwards: a
+// step then begins with the bricks that the step before it touched last, which L2 still holds; in one fixed order
+// such a state evicts itself before it comes round again.  The line is measured, half of this GPU's 126 MB of L2
+// (two partitions).  us a step, one order -> backwards on odd levels:
+//   twist FP32  42 MB 12.2 -> 12.4   64 MB 17.5 -> 17.5   85 MB 23.2 -> 23.1 (with links 24.5 -> 24.1)   106 MB 32.4 -> 29.7
+//               132 MB 44.2 -> 38.1   321 MB 117.3 -> 110.5;   FP16  66 MB 27.7 -> 27.7   161 MB 88.9 -> 84.3
+//   A-B FP32    73 MB 12.5 -> 12.0   109 MB 22.3 -> 19.2   145 MB 27.8 -> 26.7   591 MB 109.4 -> 109.0
+//       FP16    54 MB 16.7 -> 16.7   73 MB 22.4 -> 21.9   180 MB 61.6 -> 59.5   296 MB 98.2 -> 96.3
+constexpr int64_t SWEEP_BYTES = (int64_t)64 << 20;
 __device__ __forceinline__ uint32_t sweep_block(int backwards) { return backwards ? gridDim.x - 1u - blockIdx.x : blockIdx.x; }
 template <int ST, int SCHEME>
 LevelArgs with_sweep(const DomainView& v, LevelArgs a)
 {
     const int64_t arrays = SCHEME == LBM_SCHEME_ESOTERIC ? 1 : 2;
     const int64_t bytes = arrays * Q * v.n_slots * (int64_t)sizeof(typename Store<ST>::T);
-    a.backwards = (a.parity & 1) && bytes > SWEEP_BYTES && (arrays == 1 || bytes <= SWEEP_BYTES_AB);
+    a.backwards = (a.parity & 1) && bytes > SWEEP_BYTES;
     return a;
 }
 
